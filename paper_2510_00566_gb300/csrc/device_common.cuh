@@ -161,6 +161,143 @@ __device__ __forceinline__ void topk_insert_warp(unsigned long long* slots, int 
     }
 }
 
+// k above this: a flush merges a query's keys into its slots under a lock
+// (topk_merge_warp) instead of one compare-exchange chain per key.  A chain
+// costs up to k dependent global atomics (about 0.7 us each), all threads of
+// the flush side by side; a merge costs one round of loads and one of stores
+// per 128 slots whatever the number of keys, but a warp takes its queries one
+// after another.  At k = 10 the chains of a flush end sooner than eight
+// merges per warp; at k = 100 they were 84 % of the verify kernel (1.5M x 384
+// BF16, Zipf lists, 16,384 queries, k in {1, 10, 100}, with the item order of
+// inv_emit_kernel: 58.9 -> 28.2 ms a search; 1M x 768 FP8, k = 100: 31.0 ->
+// 28.5 ms).
+constexpr int kChainK = 16;
+
+// Merges up to 32 keys (one per lane, kEmptyKey = none) of one query into its
+// k ascending slots, under the query's lock; every lane of the warp calls it.
+// The slots end up as if each key had been inserted by topk_insert (an equal
+// key is kept once).  All concurrent writers of the slots must use this
+// function; readers of slots[k - 1] need no lock (slots only decrease).
+// Blocks of 128 slots are held in registers (slot 32 r + lane in v[r]); a key
+// that a block passes on (or evicts) travels to the next one.  Returns false
+// if the lock was not obtained within the wait limit.
+__device__ __forceinline__ bool topk_merge_warp(unsigned long long* slots, int k,
+                                             unsigned long long key, int* lock) {
+  const int lane = threadIdx.x & 31;
+  if (key >= ld_volatile_u64(slots + k - 1)) key = kEmptyKey;
+  uint32_t active = __ballot_sync(0xffffffffu, key != kEmptyKey);
+  if (!active) return true;
+  int got = 0;
+  if (lane == 0) {
+    const long long t0 = clock64();
+    do {
+      got = atomicCAS(lock, 0, 1) == 0;
+      if (!got) __nanosleep(64);
+    } while (!got && clock64() - t0 < kWaitCycles);
+  }
+  if (!__shfl_sync(0xffffffffu, got, 0)) return false;
+  __threadfence();
+  for (int b0 = 0; b0 < k && active; b0 += 128) {
+    const int n = k - b0 < 128 ? k - b0 : 128;
+    unsigned long long v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      v[r] = 32 * r + lane < n ? ld_volatile_u64(slots + b0 + 32 * r + lane) : kEmptyKey;
+    bool changed = false;
+    for (uint32_t m = active; m; m &= m - 1) {
+      const int j = __ffs(m) - 1;
+      const unsigned long long x = __shfl_sync(0xffffffffu, key, j);
+      int pos = 0;
+      bool dup = false;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        pos += __popc(__ballot_sync(0xffffffffu, v[r] < x));
+        dup |= v[r] == x;
+      }
+      if (__any_sync(0xffffffffu, dup)) {  // the pair is held already
+        active &= ~(1u << j);
+        continue;
+      }
+      if (pos >= n) continue;  // past this block
+      unsigned long long out = 0;  // the block's last slot is evicted
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (r == (n - 1) >> 5) out = __shfl_sync(0xffffffffu, v[r], (n - 1) & 31);
+#pragma unroll
+      for (int r = 3; r >= 0; --r) {
+        unsigned long long up = __shfl_up_sync(0xffffffffu, v[r], 1);
+        const unsigned long long wrap =
+            r > 0 ? __shfl_sync(0xffffffffu, v[r > 0 ? r - 1 : 0], 31) : 0ull;
+        if (lane == 0) up = wrap;
+        const int i = 32 * r + lane;
+        v[r] = i >= n ? kEmptyKey : (i > pos ? up : (i == pos ? x : v[r]));
+      }
+      if (lane == j) key = out;
+      if (out == kEmptyKey) active &= ~(1u << j);
+      changed = true;
+    }
+    if (changed) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (32 * r + lane < n)
+          *reinterpret_cast<volatile unsigned long long*>(slots + b0 + 32 * r + lane) = v[r];
+    }
+  }
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) atomicExch(lock, 0);
+  return true;
+}
+
+// Enters the flush's pairs into their queries' top-k: entry i < n is pair
+// list[i] (only those with sel[i] when sel is given), its distance dist[],
+// id pid[] and query pq[].  Called by all `nthreads` threads of the flush
+// (tid 0 .. nthreads - 1, n <= nthreads), between barriers.  MERGE = false:
+// every k is at most kChainK (the batch's k_max is).
+template <bool MERGE>
+__device__ __forceinline__ void topk_flush_insert(unsigned long long* topk, int k_max,
+                                                  const int32_t* __restrict__ kq, int* qlock,
+                                                  int* err, const uint16_t* list,
+                                                  const uint16_t* sel, int n, const int32_t* pq,
+                                                  const float* dist, const int32_t* pid,
+                                                  int nthreads) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < n && (!sel || sel[tid])) {
+    const int s = list[tid], q = pq[s], k = kq[q];
+    if (!MERGE || k <= kChainK)
+      topk_insert_thread(topk + (int64_t)q * k_max, k, make_key(dist[s], pid[s]));
+  }
+  if (!MERGE) return;
+  __syncwarp();
+  for (int i = tid >> 5; i < n; i += nthreads >> 5) {
+    if (sel && !sel[i]) continue;
+    const int q = pq[list[i]], k = kq[q];
+    if (k <= kChainK) continue;
+    // the warp of a query's first entry gathers all of its entries, 32 at a
+    // time (one merge site: the function is inlined where it is used, so that
+    // the flush makes no nested call, which cost the level loop registers)
+    bool mine = true;
+    int run = 0;
+    for (int base = 0; mine && (base == 0 || base < run); base += 32) {
+      unsigned long long key = kEmptyKey;
+      run = 0;
+      for (int o0 = 0; o0 < n && mine; o0 += 32) {
+        const int o = o0 + lane;
+        const uint32_t b =
+            __ballot_sync(0xffffffffu, o < n && (!sel || sel[o]) && pq[list[o]] == q);
+        if (o0 < i && (b & (i - o0 >= 32 ? 0xffffffffu : (1u << (i - o0)) - 1u))) mine = false;
+        for (uint32_t m = b; m; m &= m - 1, ++run)
+          if (lane == run - base) {
+            const int s = list[o0 + __ffs(m) - 1];
+            key = make_key(dist[s], pid[s]);
+          }
+      }
+      if (mine && !topk_merge_warp(topk + (int64_t)q * k_max, k, key, qlock + q) && lane == 0)
+        atomicOr(err, kErrTimeout);
+    }
+  }
+}
+
 // Hint that `bytes` (a multiple of 16, 16-byte aligned) at p will be read
 // soon: a bulk prefetch into L2 (no completion to wait for).
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {

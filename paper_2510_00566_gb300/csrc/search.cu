@@ -375,8 +375,13 @@ __global__ void inv_emit_kernel(int ph, const int* __restrict__ cnt, int nlist,
     int local = (int)(i - io[c]);
     int nch = (int)(chunk_off[c + 1] - chunk_off[c]);
     int nseg = (nch + seg - 1) / seg;
-    int g = local / nseg, s = local % nseg;
+    // consecutive items take different groups, each one segment further: the
+    // CTAs running together neither compete for one group's top-k slots (and
+    // prune by equally old thresholds), nor read the same slices at once (they
+    // find them in L2 an item later)
     int n_in = cnt[ph * nlist + c];
+    int ng = (n_in + qb - 1) / qb;
+    int g = local % ng, s = (local / ng + g) % nseg;
     int base = (ph == 1 ? totals[0] : 0) + bo[c] + g * qb;
     items[i] = make_int4(c, s, base, min(qb, n_in - g * qb));
   }
@@ -633,6 +638,7 @@ struct VerifyArgs {
   int* counter;
   const int32_t* bucket;
   unsigned long long* topk;
+  int* qlock;  // per query: the lock of its top-k slots (k > kChainK), zero between uses
   int* err;
   unsigned long long* stats;  // kStatWords counters (layout at kStatWords)
   int64_t items_cap;
@@ -717,7 +723,8 @@ __device__ __forceinline__ float sqrt_ratio_up(float tau, float inv_lb_up) {
 // Survivors are re-ranked in batches (those whose lower bound exceeds the
 // threshold by then are dropped); the delayed top-k insertions only leave
 // the threshold larger for a while, which is still a valid threshold.
-template <int QB, int CB, int NTH, int NST>
+// MERGE: some k of the batch is above kChainK.
+template <int QB, int CB, int NTH, int NST, bool MERGE>
 __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a) {
   constexpr int NCH = CB / CH;
   constexpr int TQ = QB / 4;
@@ -934,10 +941,9 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
       if (lane == 0) plb[s] = dist;
     }
     __syncthreads();
-    for (int i = tid; i < nk; i += NTH) {
-      const int s = keep[i], q = pq[s];
-      topk_insert_thread(a.topk + (int64_t)q * a.k_max, a.kq[q], make_key(plb[s], pid[s]));
-    }
+    for (int i0 = 0; i0 < nk; i0 += NTH)
+      topk_flush_insert<MERGE>(a.topk, a.k_max, a.kq, a.qlock, a.err, keep + i0, nullptr,
+                               min(NTH, nk - i0), pq, plb, pid, NTH);
     if (a.collect && tid == 0) s_stat[4] += nk;
   };
 
@@ -1344,7 +1350,13 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
           const int64_t slot = (tile + e / CH) * CH + (e % CH);
           const float dist =
               exact_sqdist_warp_wide(a.qorig + (int64_t)qid[g] * d, a.rows + slot * d, d);
-          topk_insert_warp(a.topk + (int64_t)qid[g] * a.k_max, qk[g], make_key(dist, ids_s[e]));
+          unsigned long long* slots = a.topk + (int64_t)qid[g] * a.k_max;
+          const unsigned long long key = make_key(dist, ids_s[e]);
+          if (!MERGE || qk[g] <= kChainK)
+            topk_insert_warp(slots, qk[g], key);
+          else if (!topk_merge_warp(slots, qk[g], lane == 0 ? key : kEmptyKey, a.qlock + qid[g]) &&
+                   lane == 0)
+            atomicOr(a.err, kErrTimeout);
         }
         if (a.collect && tid == 0) s_stat[4] += ns;
       }
@@ -1459,10 +1471,10 @@ struct TileCfg {
 constexpr TileCfg kTilesA[] = {{16, 256, 256, 3}, {16, 128, 128, 3}, {16, 64, 64, 3}};
 constexpr TileCfg kTilesB[] = {{64, 64, 256, 4}, {32, 64, 128, 4}, {16, 64, 64, 3}};
 
-template <int QB, int CB, int NTH, int NST>
+template <int QB, int CB, int NTH, int NST, bool MERGE>
 cudaError_t tile_kernel_attrs(const void** kern, size_t* static_smem) {
   static PerDeviceOnce once;
-  auto k = verify_fp32_kernel<QB, CB, NTH, NST>;
+  auto k = verify_fp32_kernel<QB, CB, NTH, NST, MERGE>;
   cudaError_t err = once.run([&] {
     cudaError_t e = allow_dynamic_smem((const void*)k);
     if (e == cudaSuccess)
@@ -1476,12 +1488,18 @@ cudaError_t tile_kernel_attrs(const void** kern, size_t* static_smem) {
   return err;
 }
 
-cudaError_t tile_attrs(const TileCfg& c, const void** kern, size_t* static_smem) {
-  if (c.QB == 16 && c.CB == 256) return tile_kernel_attrs<16, 256, 256, 3>(kern, static_smem);
-  if (c.QB == 16 && c.CB == 128) return tile_kernel_attrs<16, 128, 128, 3>(kern, static_smem);
-  if (c.QB == 64) return tile_kernel_attrs<64, 64, 256, 4>(kern, static_smem);
-  if (c.QB == 32) return tile_kernel_attrs<32, 64, 128, 4>(kern, static_smem);
-  return tile_kernel_attrs<16, 64, 64, 3>(kern, static_smem);
+template <bool MERGE>
+cudaError_t tile_attrs_of(const TileCfg& c, const void** kern, size_t* static_smem) {
+  if (c.QB == 16 && c.CB == 256) return tile_kernel_attrs<16, 256, 256, 3, MERGE>(kern, static_smem);
+  if (c.QB == 16 && c.CB == 128) return tile_kernel_attrs<16, 128, 128, 3, MERGE>(kern, static_smem);
+  if (c.QB == 64) return tile_kernel_attrs<64, 64, 256, 4, MERGE>(kern, static_smem);
+  if (c.QB == 32) return tile_kernel_attrs<32, 64, 128, 4, MERGE>(kern, static_smem);
+  return tile_kernel_attrs<16, 64, 64, 3, MERGE>(kern, static_smem);
+}
+
+cudaError_t tile_attrs(const TileCfg& c, bool merge, const void** kern, size_t* static_smem) {
+  return merge ? tile_attrs_of<true>(c, kern, static_smem)
+               : tile_attrs_of<false>(c, kern, static_smem);
 }
 
 // First tile of `list` whose stage buffers fit (blocks per SM in *bps).
@@ -1493,7 +1511,7 @@ int pick_tile(const TileCfg* list, int n, int max_w, int L, TileCfg* out, int* b
   for (int i = 0; i < n; ++i) {
     const void* k = nullptr;
     size_t ss = 0;
-    PANO_CUDA(tile_attrs(list[i], &k, &ss));
+    PANO_CUDA(tile_attrs(list[i], false, &k, &ss));  // (the same static shared memory)
     const size_t smem = FpSmem(list[i].QB, list[i].CB, max_w, L, list[i].NST).total;
     const long two = (long)per_sm / 2 - 1024 - (long)ss, one = (long)optin - (long)ss;
     const int b = (long)smem <= two ? 2 : ((long)smem <= one ? 1 : 0);
@@ -1512,7 +1530,7 @@ int pick_tile(const TileCfg* list, int n, int max_w, int L, TileCfg* out, int* b
 int launch_verify(const VerifyArgs& a, const TileCfg& c, int bps, cudaStream_t st) {
   const void* k = nullptr;
   size_t ss = 0;
-  PANO_CUDA(tile_attrs(c, &k, &ss));
+  PANO_CUDA(tile_attrs(c, a.k_max > kChainK, &k, &ss));
   int dev = 0, sms = 0;
   PANO_CUDA(cudaGetDevice(&dev));
   PANO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1778,7 +1796,10 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     }
     PANO_CUDA(cudaGetLastError());
-    // a4-a10
+    // a4-a10 (the probe stage is over: its query norms' words become the
+    // locks of the queries' top-k slots)
+    int* qlock = reinterpret_cast<int*>(qn2);
+    if (k_max > kChainK) PANO_CUDA(cudaMemsetAsync(qlock, 0, (size_t)nq * 4, st));
     if (tcpath) {
       VerifyTCArgs ta;
       std::memset(&ta, 0, sizeof(ta));
@@ -1798,6 +1819,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       ta.kq = kq;
       ta.tau_seed = tau_seed;
       ta.topk = topk;
+      ta.qlock = qlock;
       ta.err = err;
       ta.stats = stats;
       ta.d = d;
@@ -1863,6 +1885,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     va.kq = kq;
     va.tau_seed = tau_seed;
     va.topk = topk;
+    va.qlock = qlock;
     va.err = err;
     va.stats = stats;
     va.d = d;

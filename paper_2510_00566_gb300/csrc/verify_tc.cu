@@ -269,10 +269,11 @@ struct Smem {
 // moment and against each other (below); the rest get their exact distance
 // and top-k insertion, in two passes: first each query's k kept pairs of
 // smallest lower bound (ties by entry), whose exact distances usually set
-// its threshold, then the others that still pass the threshold.  All threads
+// its threshold, then the others that still pass the threshold.  All
 // epilogue threads call it (one thread per entry at most: kPend <= NE); kept out of
 // line so that it does not add to the level loop's registers.  Returns the
 // number re-ranked (thread 0; 0 elsewhere).
+template <bool MERGE>
 __device__ __noinline__ int flush_pending(const VerifyTCArgs& a, int np,
                                           const int64_t* __restrict__ pslot,
                                           const int32_t* __restrict__ pq,
@@ -321,8 +322,12 @@ __device__ __noinline__ int flush_pending(const VerifyTCArgs& a, int np,
   }
   epi_sync();
   // exact distances (a warp each; they replace the lower bounds), then the
-  // top-k insertions (a thread each, so their chains overlap)
-  auto rerank = [&](const uint16_t* list, int n, const uint16_t* sel) {
+  // top-k insertions: the pairs ranked first, then the others that still pass
+  // the thresholds of the moment
+  const uint16_t* list = keep;
+  const uint16_t* sel = rank;
+  int n = nk;
+  for (int pass = 0;; ++pass) {
     for (int i = warp; i < n; i += nw) {
       if (sel && !sel[i]) continue;
       const int s = list[i];
@@ -331,20 +336,18 @@ __device__ __noinline__ int flush_pending(const VerifyTCArgs& a, int np,
       if ((tid & 31) == 0) plb[s] = dist;
     }
     epi_sync();
-    if (tid < n && (!sel || sel[tid])) {
-      const int s = list[tid], q = pq[s];
-      topk_insert_thread(a.topk + (int64_t)q * a.k_max, a.kq[q], make_key(plb[s], pid[s]));
+    topk_flush_insert<MERGE>(a.topk, a.k_max, a.kq, a.qlock, a.err, list, sel, n, pq, plb, pid, NE);
+    epi_sync();
+    if (pass) break;
+    if (tid < nk && !first) {  // rank now lists the others
+      const int s = keep[tid], q = pq[s];
+      if (!(plb[s] > tau_of(q, a.kq[q]))) rank[atomicAdd(&s_cnt[2], 1)] = (uint16_t)s;
     }
     epi_sync();
-  };
-  rerank(keep, nk, rank);
-  // the others, against the thresholds of the moment (rank now lists them)
-  if (tid < nk && !first) {
-    const int s = keep[tid], q = pq[s];
-    if (!(plb[s] > tau_of(q, a.kq[q]))) rank[atomicAdd(&s_cnt[2], 1)] = (uint16_t)s;
+    list = rank;
+    sel = nullptr;
+    n = s_cnt[2];
   }
-  epi_sync();
-  rerank(rank, s_cnt[2], nullptr);
   return tid == 0 ? s_cnt[1] + s_cnt[2] : 0;
 }
 
@@ -361,7 +364,9 @@ __device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t& bits, int b,
 // width), kind::f8f6f4 MMAs with the query split into three E4M3 terms at one
 // power-of-two scale per group; the accumulator times the row's factor
 // s_x / (group scale) is the partial product.
-template <bool FP8>
+// MERGE: some k of the batch is above kChainK (the merges of the flush cost
+// the level loop registers, so a batch without them runs without their code).
+template <bool FP8, bool MERGE>
 __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const VerifyTCArgs a) {
   constexpr int EB = FP8 ? 1 : 2;  // bytes per stored element
   extern __shared__ unsigned char smem_raw[];
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const VerifyTCArgs a) 
     qtau[g] = tau;
   };
   auto rerank_pending = [&](int np) {
-    const int nk = flush_pending(a, np, pslot, pq, pid, plb, pub, keep, rnk, s_flush);
+    const int nk = flush_pending<MERGE>(a, np, pslot, pq, pid, plb, pub, keep, rnk, s_flush);
     if (a.collect && tid == 0) s_stat[4] += nk;
   };
   auto chunk_live = [&](int c) {
@@ -1096,7 +1101,9 @@ int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
       e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    for (const void* k : {(const void*)verify_tc_kernel<false>, (const void*)verify_tc_kernel<true>}) {
+    for (const void* k :
+         {(const void*)verify_tc_kernel<false, false>, (const void*)verify_tc_kernel<false, true>,
+          (const void*)verify_tc_kernel<true, false>, (const void*)verify_tc_kernel<true, true>}) {
       cudaFuncAttributes fa;
       if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
       if (e == cudaSuccess)
@@ -1119,10 +1126,10 @@ int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st) {
   // memory carveout, which switches only when a launch asks for more.  A
   // persistent CTA that cannot be resident yet starts later and finds the
   // queue drained, so over-provisioning is harmless.
-  if (a.fp8)
-    verify_tc_kernel<true><<<sms * 2, NT, smem, st>>>(a);
-  else
-    verify_tc_kernel<false><<<sms * 2, NT, smem, st>>>(a);
+  const bool merge = a.k_max > kChainK;
+  auto kern = a.fp8 ? (merge ? verify_tc_kernel<true, true> : verify_tc_kernel<true, false>)
+                    : (merge ? verify_tc_kernel<false, true> : verify_tc_kernel<false, false>);
+  kern<<<sms * 2, NT, smem, st>>>(a);
   PANO_CUDA(cudaGetLastError());
   return PANO_OK;
 }

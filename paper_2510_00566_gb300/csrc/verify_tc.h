@@ -32,6 +32,7 @@ struct VerifyTCArgs {
   int* counter;
   const int32_t* bucket;
   unsigned long long* topk;
+  int* qlock;  // per query: the lock of its top-k slots (k > kChainK), zero between uses
   int* err;
   unsigned long long* stats;
   int64_t items_cap;
