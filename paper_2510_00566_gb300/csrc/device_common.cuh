@@ -161,121 +161,154 @@ __device__ __forceinline__ void topk_insert_warp(unsigned long long* slots, int 
     }
 }
 
-// k above this: a flush merges a query's keys into its slots under a lock
-// (topk_merge_warp) instead of one compare-exchange chain per key.  A chain
-// costs up to k dependent global atomics (about 0.7 us each), all threads of
-// the flush side by side; a merge costs one round of loads and one of stores
-// per 128 slots whatever the number of keys, but a warp takes its queries one
-// after another.  At k = 10 the chains of a flush end sooner than eight
-// merges per warp; at k = 100 they were 84 % of the verify kernel (1.5M x 384
-// BF16, Zipf lists, 16,384 queries, k in {1, 10, 100}, with the item order of
-// inv_emit_kernel: 58.9 -> 28.2 ms a search; 1M x 768 FP8, k = 100: 31.0 ->
-// 28.5 ms).
-constexpr int kChainK = 16;
+// A query with k above this keeps its slots unsorted: a new key replaces the
+// largest one (topk_replace_warp), and its threshold lives in tau_seed alone.
+// With sorted slots a key costs up to k dependent global atomics (about 0.7 us
+// each); a replacement costs one round of loads and one of compare-exchanges
+// for up to 32 keys of a query.  At k = 10 the chains of a flush end sooner (a
+// warp takes its queries one after another); at k = 100 they were 84 % of the
+// verify kernel (1.5M x 384 BF16, Zipf lists, 16,384 queries, k in {1, 10,
+// 100}: 59 ms a search, 28 with a locked merge per flush, 20 so).  At k = 37
+// both take the same time.
+constexpr int kChainK = 40;
 
-// Merges up to 32 keys (one per lane, kEmptyKey = none) of one query into its
-// k ascending slots, under the query's lock; every lane of the warp calls it.
-// The slots end up as if each key had been inserted by topk_insert (an equal
-// key is kept once).  All concurrent writers of the slots must use this
-// function; readers of slots[k - 1] need no lock (slots only decrease).
-// Blocks of 128 slots are held in registers (slot 32 r + lane in v[r]); a key
-// that a block passes on (or evicts) travels to the next one.  Returns false
-// if the lock was not obtained within the wait limit.
-__device__ __forceinline__ bool topk_merge_warp(unsigned long long* slots, int k,
-                                             unsigned long long key, int* lock) {
+// The k-th key of a query's sorted slots, kEmptyKey where they are unsorted.
+__device__ __forceinline__ unsigned long long kth_key(const unsigned long long* slots, int k) {
+  return k <= kChainK ? ld_volatile_u64(slots + k - 1) : kEmptyKey;
+}
+
+// Smallest / largest 64-bit value of the warp.
+__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
+  const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32));
+  const uint32_t lo =
+      __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0xffffffffu);
+  return (unsigned long long)hi << 32 | lo;
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32));
+  const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : 0u);
+  return (unsigned long long)hi << 32 | lo;
+}
+
+// Enters up to 32 keys (one per lane, kEmptyKey = none) of one query into its
+// k unsorted slots (k > kChainK); every lane of the warp calls it.  Once all
+// concurrent calls have ended the slots hold the k smallest keys ever entered
+// (an equal key is kept once).
+//
+// The slots are read (128 at most in registers; more in rounds, one key at a
+// time), the keys ascending are given the slots descending while a key is
+// below its slot, and all compare-exchanges go out at once; what fails (the
+// slot was lowered meanwhile) is tried again on fresh slots.  A slot that is
+// evicted while another one above it was refilled concurrently is no loss:
+// slots only decrease, so at most as many slots above it remain as this call
+// has smaller keys, each of which still takes the largest slot of its time or
+// finds all slots below itself.
+//
+// The largest slot of what was read bounds the k-th distance from above (it can
+// only have fallen since): tau, a pointer to the query's threshold, is lowered
+// to it.
+__device__ __forceinline__ void topk_replace_warp(unsigned long long* slots, int k,
+                                                  unsigned long long key, float* tau) {
   const int lane = threadIdx.x & 31;
-  if (key >= ld_volatile_u64(slots + k - 1)) key = kEmptyKey;
-  uint32_t active = __ballot_sync(0xffffffffu, key != kEmptyKey);
-  if (!active) return true;
-  int got = 0;
-  if (lane == 0) {
-    const long long t0 = clock64();
-    do {
-      got = atomicCAS(lock, 0, 1) == 0;
-      if (!got) __nanosleep(64);
-    } while (!got && clock64() - t0 < kWaitCycles);
-  }
-  if (!__shfl_sync(0xffffffffu, got, 0)) return false;
-  __threadfence();
-  for (int b0 = 0; b0 < k && active; b0 += 128) {
-    const int n = k - b0 < 128 ? k - b0 : 128;
-    unsigned long long v[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      v[r] = 32 * r + lane < n ? ld_volatile_u64(slots + b0 + 32 * r + lane) : kEmptyKey;
-    bool changed = false;
-    for (uint32_t m = active; m; m &= m - 1) {
-      const int j = __ffs(m) - 1;
-      const unsigned long long x = __shfl_sync(0xffffffffu, key, j);
-      int pos = 0;
+  while (true) {
+    if (!__any_sync(0xffffffffu, key != kEmptyKey)) return;
+    int at = -1;  // this lane's slot
+    unsigned long long was = 0, top = 0;
+    if (k <= 128) {
+      unsigned long long v[4];
       bool dup = false;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        pos += __popc(__ballot_sync(0xffffffffu, v[r] < x));
-        dup |= v[r] == x;
+      for (int r = 0; r < 4; ++r)
+        v[r] = 32 * r + lane < k ? ld_volatile_u64(slots + 32 * r + lane) : 0ull;
+      // (an absent slot is 0: below every key, never the largest while k > 0)
+      for (uint32_t m = __ballot_sync(0xffffffffu, key != kEmptyKey); m; m &= m - 1) {
+        const unsigned long long x = __shfl_sync(0xffffffffu, key, __ffs(m) - 1);
+        const bool same = v[0] == x || v[1] == x || v[2] == x || v[3] == x;
+        if (__any_sync(0xffffffffu, same) && lane == __ffs(m) - 1) dup = true;
       }
-      if (__any_sync(0xffffffffu, dup)) {  // the pair is held already
-        active &= ~(1u << j);
+      if (dup) key = kEmptyKey;  // the pair is held already
+      bool left = key != kEmptyKey;
+      while (true) {
+        unsigned long long mx = v[0];
+        int r = 0;
+#pragma unroll
+        for (int u = 1; u < 4; ++u)
+          if (v[u] > mx) mx = v[u], r = u;
+        top = warp_max_u64(mx);
+        const unsigned long long x = warp_min_u64(left ? key : kEmptyKey);
+        if (x >= top) break;
+        const int owner = __ffs(__ballot_sync(0xffffffffu, mx == top)) - 1;
+        const int slot = __shfl_sync(0xffffffffu, 32 * r + lane, owner);
+        if (left && key == x) {  // (keys of one call are distinct: one lane)
+          at = slot;
+          was = top;
+          left = false;
+        }
+        if (lane == owner) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (u == r) v[u] = x;
+        }
+      }
+      if (left) key = kEmptyKey;  // not below any slot
+    } else {
+      // the largest slot, for the smallest key
+      unsigned long long mx = 0, x = warp_min_u64(key);
+      int i_mx = 0;
+      bool same = false;
+      for (int i = lane; i < k; i += 32) {
+        const unsigned long long v = ld_volatile_u64(slots + i);
+        same |= v == x;
+        if (v > mx) mx = v, i_mx = i;
+      }
+      top = warp_max_u64(mx);
+      const int owner = __ffs(__ballot_sync(0xffffffffu, mx == top)) - 1;
+      const int slot = __shfl_sync(0xffffffffu, i_mx, owner);
+      if (__any_sync(0xffffffffu, same)) {
+        if (key == x) key = kEmptyKey;
         continue;
       }
-      if (pos >= n) continue;  // past this block
-      unsigned long long out = 0;  // the block's last slot is evicted
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        if (r == (n - 1) >> 5) out = __shfl_sync(0xffffffffu, v[r], (n - 1) & 31);
-#pragma unroll
-      for (int r = 3; r >= 0; --r) {
-        unsigned long long up = __shfl_up_sync(0xffffffffu, v[r], 1);
-        const unsigned long long wrap =
-            r > 0 ? __shfl_sync(0xffffffffu, v[r > 0 ? r - 1 : 0], 31) : 0ull;
-        if (lane == 0) up = wrap;
-        const int i = 32 * r + lane;
-        v[r] = i >= n ? kEmptyKey : (i > pos ? up : (i == pos ? x : v[r]));
+      if (x >= top) return;
+      if (key == x) {
+        at = slot;
+        was = top;
       }
-      if (lane == j) key = out;
-      if (out == kEmptyKey) active &= ~(1u << j);
-      changed = true;
     }
-    if (changed) {
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-        if (32 * r + lane < n)
-          *reinterpret_cast<volatile unsigned long long*>(slots + b0 + 32 * r + lane) = v[r];
-    }
+    if (top != kEmptyKey && lane == 0)
+      atomicMin(reinterpret_cast<unsigned int*>(tau),
+                __float_as_uint(__fmul_ru(key_dist(top), 1.000001f)));
+    if (at >= 0 && atomicCAS(slots + at, was, key) == was) key = kEmptyKey;
+    // a lost exchange: many warps are after the same slots; spread them out
+    if (__any_sync(0xffffffffu, at >= 0 && key != kEmptyKey))
+      __nanosleep(200 + ((uint32_t)clock64() & 1023u));
   }
-  __threadfence();
-  __syncwarp();
-  if (lane == 0) atomicExch(lock, 0);
-  return true;
 }
 
 // Enters the flush's pairs into their queries' top-k: entry i < n is pair
-// list[i] (only those with sel[i] when sel is given), its distance dist[],
-// id pid[] and query pq[].  Called by all `nthreads` threads of the flush
-// (tid 0 .. nthreads - 1, n <= nthreads), between barriers.  MERGE = false:
-// every k is at most kChainK (the batch's k_max is).
-template <bool MERGE>
+// list[i], its distance dist[], id pid[] and query pq[].  Called by all
+// `nthreads` threads of the flush (tid 0 .. nthreads - 1, n <= nthreads),
+// between barriers.  LARGE = false: every k is at most kChainK (the batch's
+// k_max is).
+template <bool LARGE>
 __device__ __forceinline__ void topk_flush_insert(unsigned long long* topk, int k_max,
-                                                  const int32_t* __restrict__ kq, int* qlock,
-                                                  int* err, const uint16_t* list,
-                                                  const uint16_t* sel, int n, const int32_t* pq,
+                                                  const int32_t* __restrict__ kq, float* tau_seed,
+                                                  const uint16_t* list, int n, const int32_t* pq,
                                                   const float* dist, const int32_t* pid,
                                                   int nthreads) {
   const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < n && (!sel || sel[tid])) {
+  if (tid < n) {
     const int s = list[tid], q = pq[s], k = kq[q];
-    if (!MERGE || k <= kChainK)
+    if (!LARGE || k <= kChainK)
       topk_insert_thread(topk + (int64_t)q * k_max, k, make_key(dist[s], pid[s]));
   }
-  if (!MERGE) return;
+  if (!LARGE) return;
   __syncwarp();
   for (int i = tid >> 5; i < n; i += nthreads >> 5) {
-    if (sel && !sel[i]) continue;
     const int q = pq[list[i]], k = kq[q];
     if (k <= kChainK) continue;
     // the warp of a query's first entry gathers all of its entries, 32 at a
-    // time (one merge site: the function is inlined where it is used, so that
-    // the flush makes no nested call, which cost the level loop registers)
+    // time (one call site: inlined where it is used, so that the flush makes
+    // no nested call, which cost the level loop registers)
     bool mine = true;
     int run = 0;
     for (int base = 0; mine && (base == 0 || base < run); base += 32) {
@@ -283,8 +316,7 @@ __device__ __forceinline__ void topk_flush_insert(unsigned long long* topk, int 
       run = 0;
       for (int o0 = 0; o0 < n && mine; o0 += 32) {
         const int o = o0 + lane;
-        const uint32_t b =
-            __ballot_sync(0xffffffffu, o < n && (!sel || sel[o]) && pq[list[o]] == q);
+        const uint32_t b = __ballot_sync(0xffffffffu, o < n && pq[list[o]] == q);
         if (o0 < i && (b & (i - o0 >= 32 ? 0xffffffffu : (1u << (i - o0)) - 1u))) mine = false;
         for (uint32_t m = b; m; m &= m - 1, ++run)
           if (lane == run - base) {
@@ -292,8 +324,7 @@ __device__ __forceinline__ void topk_flush_insert(unsigned long long* topk, int 
             key = make_key(dist[s], pid[s]);
           }
       }
-      if (mine && !topk_merge_warp(topk + (int64_t)q * k_max, k, key, qlock + q) && lane == 0)
-        atomicOr(err, kErrTimeout);
+      if (mine) topk_replace_warp(topk + (int64_t)q * k_max, k, key, tau_seed + q);
     }
   }
 }

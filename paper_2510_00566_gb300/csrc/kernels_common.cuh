@@ -135,6 +135,101 @@ __device__ __forceinline__ float exact_sqdist_warp_wide(const float* __restrict_
   return s - c;
 }
 
+// Two FP32 operations per instruction (each half rounds as its scalar form).
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo2(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t x, uint64_t y, uint64_t z) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t x, uint64_t y) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t x, uint64_t y) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t x, uint64_t y) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  return r;
+}
+
+// exact_sqdist_warp_wide of two pairs at once: the same sums in the same order
+// (the same bits), one pair in each half of packed FP32 operations, so that
+// two pairs' loads and dependent sums overlap.  A flush's distances wait on
+// latency, not on arithmetic.
+__device__ __forceinline__ void exact_sqdist_warp_pair(const float* __restrict__ a0,
+                                                       const float* __restrict__ b0,
+                                                       const float* __restrict__ a1,
+                                                       const float* __restrict__ b1, int d,
+                                                       float& out0, float& out1) {
+  const int lane = threadIdx.x & 31;
+  if ((d & 3) != 0 || ((reinterpret_cast<uintptr_t>(a0) | reinterpret_cast<uintptr_t>(b0) |
+                        reinterpret_cast<uintptr_t>(a1) | reinterpret_cast<uintptr_t>(b1)) & 15)) {
+    out0 = exact_sqdist_warp_wide(a0, b0, d);
+    out1 = exact_sqdist_warp_wide(a1, b1, d);
+    return;
+  }
+  // Kahan sums of the even and odd elements; the compensations negated, so
+  // that a term is y = fma(t, t, -c)
+  uint64_t s0 = 0, n0 = 0, s1 = 0, n1 = 0;
+  auto add = [](float t, float u, uint64_t& s, uint64_t& n) {
+    const uint64_t v = pack2(t, u), y = fma2(v, v, n), w = add2(s, y);
+    n = sub2(y, sub2(w, s));
+    s = w;
+  };
+  const int d4 = d >> 2, blocks = (d4 + 255) / 256 * 4;  // (the wide form's 8-load rounds)
+  const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+  for (int i = 0; i < blocks; ++i) {
+    float4 av[2], bv[2], cv[2], dv[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int j = lane + 32 * (2 * i + u);
+      const bool in = j < d4;
+      av[u] = in ? reinterpret_cast<const float4*>(a0)[j] : z;
+      bv[u] = in ? reinterpret_cast<const float4*>(b0)[j] : z;
+      cv[u] = in ? reinterpret_cast<const float4*>(a1)[j] : z;
+      dv[u] = in ? reinterpret_cast<const float4*>(b1)[j] : z;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      add(av[u].x - bv[u].x, cv[u].x - dv[u].x, s0, n0);
+      add(av[u].y - bv[u].y, cv[u].y - dv[u].y, s1, n1);
+      add(av[u].z - bv[u].z, cv[u].z - dv[u].z, s0, n0);
+      add(av[u].w - bv[u].w, cv[u].w - dv[u].w, s1, n1);
+    }
+  }
+  // TwoSum of the s parts, the compensations and the error term summed plainly
+  auto join = [](uint64_t x, uint64_t nx, uint64_t y, uint64_t ny, uint64_t& s, uint64_t& n) {
+    const uint64_t t = add2(x, y), bb = sub2(t, x);
+    const uint64_t err = add2(sub2(x, sub2(t, bb)), sub2(y, bb));
+    n = add2(add2(nx, ny), err);
+    s = t;
+  };
+  uint64_t s, n;
+  join(s0, n0, s1, n1, s, n);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const uint64_t so = __shfl_xor_sync(0xffffffffu, (unsigned long long)s, off);
+    const uint64_t no = __shfl_xor_sync(0xffffffffu, (unsigned long long)n, off);
+    join(s, n, so, no, s, n);
+  }
+  s = add2(s, n);
+  out0 = lo2(s);
+  out1 = hi2(s);
+}
+
 // k-th smallest of the nv FP32 values vals[0..nv) (non-negative, +inf for
 // absent entries) by one warp: binary search on the bit pattern for the
 // least t with #{v <= t} >= k.  Returns +inf when fewer than k are finite.

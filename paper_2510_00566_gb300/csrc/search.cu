@@ -24,6 +24,7 @@
 #include "kernels_common.cuh"
 #include "probe_tc.h"
 #include "search.h"
+#include "tcgen05.cuh"
 #include "verify_tc.h"
 
 namespace pano {
@@ -51,10 +52,49 @@ __device__ __forceinline__ int64_t imin64(int64_t a, int64_t b) { return a < b ?
 constexpr int kNormRows = 8;      // queries (warps) per CTA
 constexpr int kNormMaxD = 1536;   // staged row length (48 KB per CTA); longer rows read global memory
 
+// What becomes of the transformed rows once their norms are taken: they stay,
+// or their place (4 d bytes) takes the tensor-core path's split image, bf16 hi
+// [d] and lo [d] or three E4M3 terms [d] at the row's power-of-two scale.
+// (Built once per query here; the verify kernel's work items, hundreds per
+// query, only copy it.)
+enum Split { kSplitNone = 0, kSplitBf16 = 1, kSplitE4m3 = 2 };
+
+// The split of elements j .. j + 7 of a row x (d % 8 == 0, x in shared
+// memory) into its place `img`.
+__device__ __forceinline__ void split8(const float* x, int j, int d, int split, float inv,
+                                       unsigned char* img) {
+  if (split == kSplitBf16) {
+    __align__(16) __nv_bfloat16 hi[8], lo[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) tc::split_bf16(x[j + u], hi[u], lo[u]);
+    *reinterpret_cast<uint4*>(img + 2 * j) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(img + 2 * (size_t)d + 2 * j) = *reinterpret_cast<const uint4*>(lo);
+  } else {
+    __align__(8) uint8_t t0[8], t1[8], t2[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) tc::split3_e4m3(x[j + u] * inv, t0[u], t1[u], t2[u]);
+    *reinterpret_cast<uint2*>(img + j) = *reinterpret_cast<const uint2*>(t0);
+    *reinterpret_cast<uint2*>(img + (size_t)d + j) = *reinterpret_cast<const uint2*>(t1);
+    *reinterpret_cast<uint2*>(img + 2 * (size_t)d + j) = *reinterpret_cast<const uint2*>(t2);
+  }
+}
+
+// The split of rows longer than kNormMaxD (one CTA per row, staged whole).
+__global__ void __launch_bounds__(256) split_rows_kernel(float* qt, int d, int split,
+                                                         const float4* __restrict__ qinfo) {
+  extern __shared__ float srow[];
+  float* x = qt + (int64_t)blockIdx.x * d;
+  for (int j = threadIdx.x; j < d; j += blockDim.x) srow[j] = x[j];
+  __syncthreads();
+  const float inv = ldexpf(1.f, -min(60, tc::e4m3_exponent(qinfo[blockIdx.x].w)));
+  for (int j = 8 * threadIdx.x; j < d; j += 8 * blockDim.x)
+    split8(srow, j, d, split, inv, reinterpret_cast<unsigned char*>(x));
+}
+
 __global__ void __launch_bounds__(kNormRows * 32) query_norms_kernel(
-    const float* __restrict__ q, const float* __restrict__ qt, int64_t nq, int d, int L,
+    const float* __restrict__ q, float* qt, int64_t nq, int d, int L,
     const int32_t* __restrict__ level_off, const float* __restrict__ mu, float c_trans_up,
-    float4* __restrict__ qinfo, float* __restrict__ qtail, float* __restrict__ qn2) {
+    float4* __restrict__ qinfo, float* __restrict__ qtail, float* __restrict__ qn2, int split) {
   extern __shared__ float qrow_s[];  // [kNormRows][d] when d <= kNormMaxD
   const int w = threadIdx.x / 32, lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * kNormRows + w;
@@ -96,6 +136,11 @@ __global__ void __launch_bounds__(kNormRows * 32) query_norms_kernel(
     qinfo[row] = make_float4(nqf, sqrtf(nqf),
                              __fmul_ru(c_trans_up, __fsqrt_ru(acc2_upper(dev, 0x1p-21f))), xmax);
     qn2[row] = __fadd_rn(on.s, on.c);
+  }
+  if (split != kSplitNone && d <= kNormMaxD) {  // the staged row goes back split
+    const float inv = ldexpf(1.f, -min(60, tc::e4m3_exponent(xmax)));
+    for (int j = 8 * lane; j < d; j += 256)
+      split8(x, j, d, split, inv, reinterpret_cast<unsigned char*>(qt + row * d));
   }
 }
 
@@ -388,7 +433,7 @@ __global__ void inv_emit_kernel(int ph, const int* __restrict__ cnt, int nlist,
 }
 
 // ------------------------------------------------- Alg. 1 warm start (a6)
-// Per query: distances to the first max(4k, 64) (at most 256) members of its
+// Per query: distances to the first max(4k, 64) (at most 512) members of its
 // nearest list; the k-th smallest is an upper bound on d_k and seeds the
 // threshold before any tile is verified.  Algorithm 1 also fills its heap
 // with k candidates before pruning anything; that matters once the
@@ -407,7 +452,7 @@ __global__ void inv_emit_kernel(int ph, const int* __restrict__ cnt, int nlist,
 // computed one times 1 / ((1 - gamma_m)(1 - u)^2) <= slack = 1 + 2(m + 3)u
 // (host-computed, rounded up); multiplying by it (rounding up) keeps every
 // seed distance an upper bound on the exact one.
-constexpr int kSeedMax = 256;
+constexpr int kSeedMax = 512;
 constexpr int kSeedWarps = 8;
 
 __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
@@ -638,7 +683,6 @@ struct VerifyArgs {
   int* counter;
   const int32_t* bucket;
   unsigned long long* topk;
-  int* qlock;  // per query: the lock of its top-k slots (k > kChainK), zero between uses
   int* err;
   unsigned long long* stats;  // kStatWords counters (layout at kStatWords)
   int64_t items_cap;
@@ -723,8 +767,8 @@ __device__ __forceinline__ float sqrt_ratio_up(float tau, float inv_lb_up) {
 // Survivors are re-ranked in batches (those whose lower bound exceeds the
 // threshold by then are dropped); the delayed top-k insertions only leave
 // the threshold larger for a while, which is still a valid threshold.
-// MERGE: some k of the batch is above kChainK.
-template <int QB, int CB, int NTH, int NST, bool MERGE>
+// LARGE: some k of the batch is above kChainK.
+template <int QB, int CB, int NTH, int NST, bool LARGE>
 __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a) {
   constexpr int NCH = CB / CH;
   constexpr int TQ = QB / 4;
@@ -889,7 +933,7 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
   auto read_tau = [&](int g, int G) {
     TauRead r{kEmptyKey, -1.f};  // k == 0: nothing can enter
     if (g < G && qk[g] > 0) {
-      r.key = ld_volatile_u64(a.topk + (int64_t)qid[g] * a.k_max + qk[g] - 1);
+      r.key = kth_key(a.topk + (int64_t)qid[g] * a.k_max, qk[g]);
       r.seed = __ldcg(a.tau_seed + qid[g]);
     }
     return r;
@@ -912,7 +956,7 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
     // k are closer; the pair's own upper bound is never below its lower one)
     for (int s = tid; s < np; s += NTH) {
       const int q = pq[s], kk = a.kq[q];
-      const unsigned long long key = ld_volatile_u64(a.topk + (int64_t)q * a.k_max + kk - 1);
+      const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, kk);
       const float tau = fminf(key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f),
                               __ldcg(a.tau_seed + q));
       const float lb = plb[s];
@@ -942,7 +986,7 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
     }
     __syncthreads();
     for (int i0 = 0; i0 < nk; i0 += NTH)
-      topk_flush_insert<MERGE>(a.topk, a.k_max, a.kq, a.qlock, a.err, keep + i0, nullptr,
+      topk_flush_insert<LARGE>(a.topk, a.k_max, a.kq, a.tau_seed, keep + i0,
                                min(NTH, nk - i0), pq, plb, pid, NTH);
     if (a.collect && tid == 0) s_stat[4] += nk;
   };
@@ -1352,11 +1396,10 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
               exact_sqdist_warp_wide(a.qorig + (int64_t)qid[g] * d, a.rows + slot * d, d);
           unsigned long long* slots = a.topk + (int64_t)qid[g] * a.k_max;
           const unsigned long long key = make_key(dist, ids_s[e]);
-          if (!MERGE || qk[g] <= kChainK)
+          if (!LARGE || qk[g] <= kChainK)
             topk_insert_warp(slots, qk[g], key);
-          else if (!topk_merge_warp(slots, qk[g], lane == 0 ? key : kEmptyKey, a.qlock + qid[g]) &&
-                   lane == 0)
-            atomicOr(a.err, kErrTimeout);
+          else
+            topk_replace_warp(slots, qk[g], lane == 0 ? key : kEmptyKey, a.tau_seed + qid[g]);
         }
         if (a.collect && tid == 0) s_stat[4] += ns;
       }
@@ -1410,7 +1453,19 @@ __global__ void decode_kernel(int64_t nq, int k_max, const int32_t* __restrict__
   if (e >= nq * k_max) return;
   int64_t qi = e / k_max;
   int j = (int)(e % k_max);
-  unsigned long long key = j < kq[qi] ? topk[e] : kEmptyKey;
+  const int k = kq[qi];
+  unsigned long long key = j < k ? topk[e] : kEmptyKey;
+  if (k > kChainK && j < k) {
+    // unsorted slots: a key's place is the number of smaller ones (keys are
+    // distinct), an empty slot's the keys plus the empty slots before it
+    const unsigned long long* slots = topk + qi * k_max;
+    int r = 0;
+    for (int i = 0; i < k; ++i) {
+      const unsigned long long o = slots[i];
+      r += o < key || (o == kEmptyKey && key == kEmptyKey && i < j);
+    }
+    e += r - j;
+  }
   if (key == kEmptyKey) {
     out_ids[e] = -1;
     out_d[e] = INFINITY;
@@ -1471,10 +1526,10 @@ struct TileCfg {
 constexpr TileCfg kTilesA[] = {{16, 256, 256, 3}, {16, 128, 128, 3}, {16, 64, 64, 3}};
 constexpr TileCfg kTilesB[] = {{64, 64, 256, 4}, {32, 64, 128, 4}, {16, 64, 64, 3}};
 
-template <int QB, int CB, int NTH, int NST, bool MERGE>
+template <int QB, int CB, int NTH, int NST, bool LARGE>
 cudaError_t tile_kernel_attrs(const void** kern, size_t* static_smem) {
   static PerDeviceOnce once;
-  auto k = verify_fp32_kernel<QB, CB, NTH, NST, MERGE>;
+  auto k = verify_fp32_kernel<QB, CB, NTH, NST, LARGE>;
   cudaError_t err = once.run([&] {
     cudaError_t e = allow_dynamic_smem((const void*)k);
     if (e == cudaSuccess)
@@ -1488,17 +1543,17 @@ cudaError_t tile_kernel_attrs(const void** kern, size_t* static_smem) {
   return err;
 }
 
-template <bool MERGE>
+template <bool LARGE>
 cudaError_t tile_attrs_of(const TileCfg& c, const void** kern, size_t* static_smem) {
-  if (c.QB == 16 && c.CB == 256) return tile_kernel_attrs<16, 256, 256, 3, MERGE>(kern, static_smem);
-  if (c.QB == 16 && c.CB == 128) return tile_kernel_attrs<16, 128, 128, 3, MERGE>(kern, static_smem);
-  if (c.QB == 64) return tile_kernel_attrs<64, 64, 256, 4, MERGE>(kern, static_smem);
-  if (c.QB == 32) return tile_kernel_attrs<32, 64, 128, 4, MERGE>(kern, static_smem);
-  return tile_kernel_attrs<16, 64, 64, 3, MERGE>(kern, static_smem);
+  if (c.QB == 16 && c.CB == 256) return tile_kernel_attrs<16, 256, 256, 3, LARGE>(kern, static_smem);
+  if (c.QB == 16 && c.CB == 128) return tile_kernel_attrs<16, 128, 128, 3, LARGE>(kern, static_smem);
+  if (c.QB == 64) return tile_kernel_attrs<64, 64, 256, 4, LARGE>(kern, static_smem);
+  if (c.QB == 32) return tile_kernel_attrs<32, 64, 128, 4, LARGE>(kern, static_smem);
+  return tile_kernel_attrs<16, 64, 64, 3, LARGE>(kern, static_smem);
 }
 
-cudaError_t tile_attrs(const TileCfg& c, bool merge, const void** kern, size_t* static_smem) {
-  return merge ? tile_attrs_of<true>(c, kern, static_smem)
+cudaError_t tile_attrs(const TileCfg& c, bool large, const void** kern, size_t* static_smem) {
+  return large ? tile_attrs_of<true>(c, kern, static_smem)
                : tile_attrs_of<false>(c, kern, static_smem);
 }
 
@@ -1716,13 +1771,20 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     mark(0);
     PANO_CUDA(gemm_nt(kStore, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(), d,
                       qt, d, nullptr, nullptr, st));
+    const int split = I.precision == PANO_BF16  ? kSplitBf16
+                      : I.precision == PANO_FP8 ? kSplitE4m3
+                                                : kSplitNone;
     float c_trans_up = (float)I.c_trans;  // rounded up: the e_q bound stays an upper bound
     if ((double)c_trans_up < I.c_trans) c_trans_up = std::nextafter(c_trans_up, INFINITY);
     query_norms_kernel<<<(unsigned)((nq + kNormRows - 1) / kNormRows), kNormRows * 32,
                          d <= kNormMaxD ? (size_t)kNormRows * d * 4 : 0, st>>>(
         queries, qt, nq, d, L, I.level_off_d.as<int32_t>(), I.mu32.as<float>(), c_trans_up, qinfo,
-        qtail, qn2);
+        qtail, qn2, split);
     PANO_CUDA(cudaGetLastError());
+    if (split != kSplitNone && d > kNormMaxD) {
+      split_rows_kernel<<<(unsigned)nq, 256, (size_t)d * 4, st>>>(qt, d, split, qinfo);
+      PANO_CUDA(cudaGetLastError());
+    }
     // a2
     mark(1);
     if (nlist > 1) {
@@ -1796,10 +1858,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     }
     PANO_CUDA(cudaGetLastError());
-    // a4-a10 (the probe stage is over: its query norms' words become the
-    // locks of the queries' top-k slots)
-    int* qlock = reinterpret_cast<int*>(qn2);
-    if (k_max > kChainK) PANO_CUDA(cudaMemsetAsync(qlock, 0, (size_t)nq * 4, st));
+    // a4-a10
     if (tcpath) {
       VerifyTCArgs ta;
       std::memset(&ta, 0, sizeof(ta));
@@ -1819,7 +1878,6 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       ta.kq = kq;
       ta.tau_seed = tau_seed;
       ta.topk = topk;
-      ta.qlock = qlock;
       ta.err = err;
       ta.stats = stats;
       ta.d = d;
@@ -1885,7 +1943,6 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     va.kq = kq;
     va.tau_seed = tau_seed;
     va.topk = topk;
-    va.qlock = qlock;
     va.err = err;
     va.stats = stats;
     va.d = d;
@@ -2065,7 +2122,7 @@ int transform_queries(const pano_index& I, const float* queries, int64_t nq, flo
   query_norms_kernel<<<(unsigned)((nq + kNormRows - 1) / kNormRows), kNormRows * 32,
                        d <= kNormMaxD ? (size_t)kNormRows * d * 4 : 0, st>>>(
       queries, qt, nq, d, L, I.level_off_d.as<int32_t>(), I.mu32.as<float>(), c_trans_up, qinfo,
-      qtail, qn2);
+      qtail, qn2, kSplitNone);
   PANO_CUDA(cudaGetLastError());
   return PANO_OK;
 }

@@ -178,6 +178,27 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 8 consecutive f32 columns (same lane rule).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// One f32 column (same lane rule).
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  return __uint_as_float(r);
+}
+
 // bf16 hi/lo split of an FP32 value: x ~= hi + lo with |x - hi - lo| <=
 // 2^-16 |x| (both round to nearest).
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
@@ -197,6 +218,15 @@ __device__ __forceinline__ float e4m3_to_f32(uint8_t b) {
   const uint32_t e = (b >> 3) & 0xfu, mm = b & 7u;
   const float m = e ? __uint_as_float(((e + 120u) << 23) | (mm << 20)) : (float)mm * 0x1p-9f;
   return (b & 0x80u) ? -m : m;
+}
+
+// Exponent e of the scale 2^e for values of magnitude at most m: m / 2^e is
+// at most 448, so no E4M3 term saturates (-60 at least: a smaller one only
+// adds underflow).
+__device__ __forceinline__ int e4m3_exponent(float m) {
+  int e = 0;
+  if (m > 0.f) frexpf(m / 448.f, &e);
+  return e < -60 ? -60 : e;
 }
 
 // Three-term E4M3 split of an FP32 value y with |y| <= 448: y ~= t0 + t1 + t2,

@@ -21,7 +21,7 @@ struct VerifyTCArgs {
   const float* xscale;  // FP8: per-vector power-of-two scale s_x
   const float* rows;
   const int64_t* chunk_off;
-  const float* qt;
+  const float* qt;  // per query (4 d bytes) its split image: bf16 hi [d], lo [d], or E4M3 terms [3][d]
   const float* qorig;
   const float4* qinfo;
   const float* qtail;
@@ -32,7 +32,6 @@ struct VerifyTCArgs {
   int* counter;
   const int32_t* bucket;
   unsigned long long* topk;
-  int* qlock;  // per query: the lock of its top-k slots (k > kChainK), zero between uses
   int* err;
   unsigned long long* stats;
   int64_t items_cap;
@@ -61,6 +60,5 @@ int launch_pack_fp8(const float* xt, const float* rows, const int64_t* perm, int
                     double c_trans, uint8_t* slices, float* tails, float* xn2, float* ex,
                     float* xscale, int32_t* ids, cudaStream_t st);
 int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st);
-size_t verify_tc_smem(int max_w, bool fp8);
 
 }  // namespace pano

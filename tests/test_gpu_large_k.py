@@ -1,6 +1,7 @@
-"""Top-k insertion at the k where it changes: up to 16 keys go in by atomic
-chains, more by warp merges over blocks of 128 slots (k at the edges of both),
-mixed in one batch, with many work items competing for each query's slots."""
+"""Top-k insertion at the k where it changes: up to 40 sorted slots are kept by
+atomic chains, more stay unsorted and a new key replaces the largest (up to 128
+slots in registers, more in rounds), mixed in one batch, with many work items
+competing for each query's slots."""
 import numpy as np
 import pytest
 import torch
@@ -23,7 +24,7 @@ def test_mixed_k_at_the_insertion_edges(precision):
     t = pano.panorama_fit_transform(X, n_levels=2)
     idx = pano.panorama_build_ivf(t, w.X.to(DEV), nlist=2, level_widths=[64, 64],
                                   precision=precision, centroids=C)
-    k = np.resize([1, 16, 17, 32, 33, 127, 128, 129, 256, 300, 1024, 0], len(Q)).astype(np.int32)
+    k = np.resize([1, 16, 33, 40, 41, 64, 127, 128, 129, 300, 1024, 0], len(Q)).astype(np.int32)
     ids, d = idx.search(torch.from_numpy(Q).to(DEV), 2, torch.from_numpy(k).to(DEV), k_max=1024)
     lists, _ = oracle.assign(X, C)
     ref = oracle.ivf_search(X, Q, C, 2, 1024, lists_of_vector=lists)
