@@ -10,14 +10,12 @@
 // ||x~||^2 and the transform error bound e_x [n], and the original rows [n][d]
 // for the exact re-ranking.  The id of a vector is its row.
 //
-// Search (refine_kernel, one CTA per query): Algorithm 1 seeds the heap with
-// the first k candidates' exact distances; the rest go in rounds of 256, one
-// candidate per thread, refined level by level against the round's
-// threshold with the margined separable test of the IVF kernels.  The
-// survivors of a round are checked against the threshold of the moment and
-// against each other (k survivors with upper bounds below a lower bound rule
-// it out), then re-ranked on the original rows (a warp each) and inserted
-// into the query's top-k in shared memory (a thread each).
+// Search (refine_kernel, one CTA per query): Algorithm 1 seeds the heap with k
+// exact distances; the rest are refined level by level, eight lanes per
+// candidate, against the threshold of the moment with the margined separable
+// test of the IVF kernels.  A candidate that passes every level is re-ranked at
+// once on the original rows by its warp and inserted into the query's top-k in
+// shared memory.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -31,7 +29,8 @@
 namespace pano {
 namespace {
 
-constexpr int RT = 256;           // threads per query: one candidate each per round
+constexpr int RT = 256;           // threads per query
+constexpr int RG = 8;             // lanes per candidate
 constexpr int RW = RT / 32;
 constexpr int kRefineMaxK = 1024;
 constexpr int kSeedScan = 2048;  // candidates ranked for the seed (shared memory)
@@ -92,11 +91,6 @@ struct RefineArgs {
   int32_t level_off[65];
 };
 
-__device__ __forceinline__ float threshold_of(const unsigned long long* topk, int k) {
-  const unsigned long long key = topk[k - 1];
-  return key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f);
-}
-
 // sqrt(tau / lb_scale) rounded up (rsqrtf: at most 2 ulp; the factor
 // 1 + 2^-19 covers it and the products' roundings).
 __device__ __forceinline__ float sqrt_ratio_up_r(float tau, float inv_lb_up) {
@@ -105,29 +99,71 @@ __device__ __forceinline__ float sqrt_ratio_up_r(float tau, float inv_lb_up) {
   return __fmul_ru(__fmul_ru(y, rsqrtf(y)), 1.0f + 0x1p-19f);
 }
 
+// Partial product of coordinates [m0, m1) of a row by the eight lanes of a
+// group (every lane of the group gets it; lanes of groups that are off pass
+// on = false and must call it too).  A group's lanes read 128 consecutive
+// bytes at a time.
+__device__ __forceinline__ float group_dot(const float* qs, const float* x, int m0, int m1,
+                                           bool vec, bool on, int t) {
+  float acc = 0.f;
+  if (on) {
+    if (vec) {
+      const float4* x4 = reinterpret_cast<const float4*>(x);
+      const float4* q4 = reinterpret_cast<const float4*>(qs);
+      const int e = m1 >> 2;
+#pragma unroll 4
+      for (int j = (m0 >> 2) + t; j < e; j += RG) {
+        const float4 xv = __ldg(x4 + j);
+        const float4 qv = q4[j];
+        acc = fmaf(qv.x, xv.x, acc);
+        acc = fmaf(qv.y, xv.y, acc);
+        acc = fmaf(qv.z, xv.z, acc);
+        acc = fmaf(qv.w, xv.w, acc);
+      }
+    } else {
+      for (int j = m0 + t; j < m1; j += RG) acc = fmaf(qs[j], __ldg(x + j), acc);
+    }
+  }
+#pragma unroll
+  for (int off = RG / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  return acc;
+}
+
+// Bound: gathered row segments (L2 / HBM): a candidate-level is one slice of a
+// scattered row.  Eight lanes per candidate read whole 128-byte lines of it (a
+// lane per row used half of every sector it fetched, one 16-byte load at a
+// time), and the four candidates of a warp go on independently: each group
+// takes its next candidate when its own dies, so no lane waits for another
+// candidate's levels and the threshold is always the current one (rounds of
+// 256 candidates ended in a block barrier each).  4,096 queries x 1,000
+// candidates of 960 coordinates, k = 10: 4.66 -> 2.23 ms.
 __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
   const int d = a.d, L = a.L, k = a.k, kp = a.kp;
+  const int ns = min(kp, kSeedScan);
   float* qs = reinterpret_cast<float*>(sm);  // q~ [d], 16-byte aligned for float4 reads
   unsigned long long* topk = reinterpret_cast<unsigned long long*>(qs + ((d + 3) & ~3));  // [k]
+  float* akey = reinterpret_cast<float*>(topk + k);  // [ns]
+  float* p0s = akey + ns;                            // [ns] first-level partial products
   __shared__ float qtl[65];
-  __shared__ int64_t pslot[RT];
-  __shared__ float plb[RT], pub[RT];
-  __shared__ uint16_t keep[RT];
-  __shared__ int s_np, s_nk;
-  __shared__ float4 s_qterm;  // (E, g rq, H_q, tau)
+  __shared__ int s_next;
+  __shared__ float s_tk;
   __shared__ unsigned long long s_dims, s_cands, s_rer;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
+  const int grp = lane / RG, t = lane % RG;
   const int64_t q = blockIdx.x;
   for (int i = tid; i < k; i += RT) topk[i] = kEmptyKey;
   for (int j = tid; j < d; j += RT) qs[j] = a.qt[q * d + j];
   for (int l = tid; l <= L; l += RT) qtl[l] = a.eps * a.qtail[q * (L + 1) + l];
-  if (tid == 0) s_dims = s_cands = s_rer = 0;
+  if (tid == 0) {
+    s_dims = s_cands = s_rer = 0;
+    s_next = 0;
+  }
   const float4 inf = a.qinfo[q];
   const float nq = inf.x, rq = inf.y, eq = inf.z, gs = a.gslack;
   const int64_t* cl = a.cand + q * (int64_t)kp;
   const float* qo = a.qorig + q * (int64_t)d;
-  const bool vec = (d & 3) == 0;
+  const bool vec_d = (d & 3) == 0;
   __syncthreads();
 
   auto valid_id = [&](int64_t id) {
@@ -141,25 +177,40 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   // is free, so they are the k of smallest approximate distance after the
   // first level, A^(1) = ||q~||^2 + ||x~||^2 - 2 p^(0,1) (>= 0: the first
   // level's squared distance plus both tail energies), among the first
-  // kSeedScan candidates.  A seed is marked -1 in akey and skipped later.
-  const int ns = min(kp, kSeedScan);
+  // kSeedScan candidates.  A seed is marked -1 in akey and skipped later; the
+  // first level's partial products are kept for the others.
   const int m1 = a.level_off[1];
-  float* akey = reinterpret_cast<float*>(topk + k);  // [ns]
-  unsigned long long dims0 = 0;
-  for (int c = tid; c < ns; c += RT) {
-    const int64_t id = cl[c];
-    float key = INFINITY;
-    if (valid_id(id)) {
-      const float* x = a.xt + id * d;
-      float p0 = 0.f;
-      for (int j = 0; j < m1; ++j) p0 = fmaf(qs[j], x[j], p0);
-      key = fmaxf(nq + a.xn2[id] - 2.f * p0, 0.f);
-      dims0 += (unsigned long long)m1;
+  const bool vec0 = vec_d && (m1 & 3) == 0;
+  unsigned long long dims = 0;  // (lane 0 of each group)
+  constexpr int GPB = RT / RG;  // groups of the block
+  for (int c0 = 0; c0 < ns; c0 += 2 * GPB) {
+    int64_t id[2];
+    bool on[2];
+    float nx[2], p0[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int c = c0 + u * GPB + warp * (32 / RG) + grp;
+      id[u] = c < ns ? cl[c] : -1;
+      on[u] = id[u] >= 0 && id[u] < a.n;
+      nx[u] = on[u] ? __ldg(a.xn2 + id[u]) : 0.f;
     }
-    akey[c] = key;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      p0[u] = group_dot(qs, a.xt + (on[u] ? id[u] : 0) * d, 0, m1, vec0, on[u], t);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int c = c0 + u * GPB + warp * (32 / RG) + grp;
+      if (c >= ns || t) continue;
+      float key = INFINITY;
+      if (valid_id(id[u])) {
+        key = fmaxf(nq + nx[u] - 2.f * p0[u], 0.f);
+        dims += (unsigned long long)m1;
+      }
+      akey[c] = key;
+      p0s[c] = p0[u];
+    }
   }
   __syncthreads();
-  __shared__ float s_tk;
   if (warp == 0) {
     const float tk = warp_kth_smallest(akey, ns, k);
     if (lane == 0) s_tk = tk;
@@ -182,99 +233,106 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
       atomicAdd(&s_dims, (unsigned long long)d);
     }
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) dims0 += __shfl_xor_sync(0xffffffffu, dims0, off);
-  if (lane == 0 && dims0) atomicAdd(&s_dims, dims0);
   __syncthreads();
 
-  for (int r0 = 0; r0 < kp; r0 += RT) {
-    if (tid == 0) {
-      s_np = 0;
-      const float tau = threshold_of(topk, k);
-      const float st = tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up);
-      const float E = __fadd_ru(eq, st);
-      s_qterm = make_float4(E, gs * rq, 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E)),
-                            tau);
-    }
-    __syncthreads();
-    const float4 t = s_qterm;
-    const int c = r0 + tid;
-    const bool seeded = c < ns && akey[c] < 0.f;
-    const int64_t id = c < kp && !seeded ? cl[c] : -1;
-    unsigned long long dims = 0;
-    if (c < kp && !seeded && valid_id(id)) {
-      const float* x = a.xt + id * d;
-      const float* tx = a.tails + id * (L + 1);
-      const float nx = a.xn2[id], rx = sqrtf(nx), exv = a.ex[id];
-      const float Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
-      float p = 0.f;
-      bool alive = true;
-      for (int l = 0; l < L && alive; ++l) {
-        const int m0 = a.level_off[l], m1 = a.level_off[l + 1];
-        float acc = 0.f;
-        if (vec && ((m0 | m1) & 3) == 0) {
-          for (int j = m0; j < m1; j += 4) {
-            const float4 xv = *reinterpret_cast<const float4*>(x + j);
-            const float4 qv = *reinterpret_cast<const float4*>(qs + j);
-            acc = fmaf(qv.x, xv.x, acc);
-            acc = fmaf(qv.y, xv.y, acc);
-            acc = fmaf(qv.z, xv.z, acc);
-            acc = fmaf(qv.w, xv.w, acc);
-          }
-        } else {
-          for (int j = m0; j < m1; ++j) acc = fmaf(qs[j], x[j], acc);
+  // The other candidates, a group of eight lanes each.
+  unsigned long long seen = kEmptyKey - 1;  // the k-th key that E and Hq stand for
+  float E = 0.f, Hq = 0.f;
+  unsigned n_cand = 0, n_rer = 0;
+  int64_t id = -1;    // the group's candidate (-1: none), its level and partial product
+  int l = 0;
+  float p = 0.f, rx = 0.f, exv = 0.f, Hx = 0.f;
+  bool open = true;   // the list is not exhausted
+  const unsigned gmask = 0xffu << (grp * RG);
+  while (true) {
+    // groups without a candidate take the next one of the list
+    if (id < 0 && open) {
+      while (true) {
+        int c = 0;
+        if (t == 0) c = atomicAdd(&s_next, 1);
+        c = __shfl_sync(gmask, c, grp * RG);
+        if (c >= kp) {
+          open = false;
+          break;
         }
-        p += acc;
-        dims += (unsigned long long)(m1 - m0);
-        // margined Eq. 3 (separable form): pruned when LB > tau
-        const float P = fmaf(t.x, exv, fmaf(t.y, rx, fmaf(qtl[l + 1], tx[l + 1], p)));
-        if (P < t.z + Hx) alive = false;
+        if (c < ns && akey[c] < 0.f) continue;  // a seed
+        const int64_t i = cl[c];
+        if (i < 0 || i >= a.n) {
+          if (t == 0) valid_id(i);
+          continue;
+        }
+        id = i;
+        const float nx = __ldg(a.xn2 + i);
+        exv = __ldg(a.ex + i);
+        rx = sqrtf(nx);
+        Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
+        l = 0;
+        p = 0.f;
+        if (t == 0) ++n_cand;
+        if (c < ns) {  // its first level is known
+          p = p0s[c];
+          l = -1;
+        }
+        break;
       }
-      if (alive) {  // its Eq. 3 bounds after the last level (C = 0)
-        const float A = nq + nx - 2.f * p, S = rq + rx;
-        const float lr = sqrtf(fmaxf(A - gs * S * S, 0.f)) - (eq + exv);
-        const float ru = __fadd_ru(__fsqrt_ru(fmaxf(A + gs * S * S, 0.f)), eq + exv);
-        const int pos = atomicAdd(&s_np, 1);
-        pslot[pos] = id;
-        plb[pos] = lr > 0.f ? lr * lr * a.lb_scale : 0.f;
-        pub[pos] = __fmul_ru(__fmul_ru(ru, ru), a.ub_scale);
+    }
+    __syncwarp();
+    const bool on = id >= 0;
+    if (!__any_sync(0xffffffffu, on)) break;
+    // (one value for the warp: the lanes of a group must decide alike)
+    const unsigned long long kth =
+        __shfl_sync(0xffffffffu, ld_volatile_u64(topk + k - 1), 0);
+    if (kth != seen) {
+      seen = kth;
+      const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
+      E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
+      Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
+    }
+    // one level of every group's candidate (a first level that is known is
+    // only tested); the next level's lines head for L2 meanwhile
+    const bool known = l < 0;
+    if (known) l = 0;
+    const int a0 = on ? a.level_off[l] : 0, a1 = on ? a.level_off[l + 1] : 0;
+    const float* x = a.xt + (on ? id : 0) * (int64_t)d;
+    float tx = 0.f;
+    if (on) {
+      tx = __ldg(a.tails + id * (L + 1) + l + 1);
+      const int nxt = a1 + 32 * t;  // (128 bytes per lane)
+      if (l + 1 < L && nxt < a.level_off[l + 2])
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(x + nxt));
+    }
+    const float s = group_dot(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, on && !known, t);
+    bool done = false;
+    if (on) {
+      if (!known) {
+        p += s;
+        if (t == 0) dims += (unsigned long long)(a1 - a0);
       }
-      atomicAdd(&s_cands, 1ull);
+      // margined Eq. 3 (separable form): pruned when LB > tau
+      const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
+      if (P < Hq + Hx)
+        id = -1;
+      else if (++l == L)
+        done = true;
     }
-    // coordinates read (one atomic per warp)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) dims += __shfl_xor_sync(0xffffffffu, dims, off);
-    if (lane == 0 && dims) atomicAdd(&s_dims, dims);
-    if (tid == 0) s_nk = 0;
-    __syncthreads();
-    // the round's survivors: dropped if above the threshold of the moment or
-    // if k survivors have upper bounds below its lower bound
-    const int np = s_np;
-    if (tid < np) {
-      const float lb = plb[tid];
-      bool keep_s = !(lb > threshold_of(topk, k));
-      if (keep_s) {
-        int below = 0;
-        for (int o = 0; o < np && below < k; ++o) below += __fmul_ru(pub[o], 1.000001f) < lb;
-        keep_s = below < k;
+    // what passed every level: its exact distance, by the whole warp
+    for (unsigned m = __ballot_sync(0xffffffffu, done && t == 0); m; m &= m - 1) {
+      const int64_t i = __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
+      const float dist = exact_sqdist_warp_wide(qo, a.rows + i * d, d);
+      if (lane == 0) {
+        topk_insert_thread(topk, k, make_key(dist, (int32_t)i));
+        ++n_rer;
       }
-      if (keep_s) keep[atomicAdd(&s_nk, 1)] = (uint16_t)tid;
+      __syncwarp();
     }
-    __syncthreads();
-    const int nk = s_nk;
-    for (int i = warp; i < nk; i += RW) {
-      const int s = keep[i];
-      const float dist = exact_sqdist_warp_wide(qo, a.rows + pslot[s] * d, d);
-      if (lane == 0) plb[s] = dist;
-    }
-    __syncthreads();
-    if (tid < nk) {
-      const int s = keep[tid];
-      topk_insert_thread(topk, k, make_key(plb[s], (int32_t)pslot[s]));
-    }
-    if (tid == 0) s_rer += (unsigned long long)nk;
-    __syncthreads();
+    if (done) id = -1;
   }
+  if (t == 0) {
+    atomicAdd(&s_dims, dims);
+    atomicAdd(&s_cands, (unsigned long long)n_cand);
+    if (lane == 0) atomicAdd(&s_rer, (unsigned long long)n_rer);
+  }
+  __syncthreads();
   for (int i = tid; i < k; i += RT) {
     const unsigned long long key = topk[i];
     a.out_ids[q * k + i] = key == kEmptyKey ? -1 : (int64_t)key_id(key);
@@ -433,7 +491,7 @@ int refine(const pano_index* ip, const float* queries, int64_t nq, const int64_t
   a.eps = epsilon > 0.f ? epsilon : 1.f;
   for (int l = 0; l <= L; ++l) a.level_off[l] = I.offs[l];
   const size_t smem =
-      (size_t)((d + 3) & ~3) * 4 + (size_t)k * 8 + (size_t)std::min(kprime, kSeedScan) * 4;
+      (size_t)((d + 3) & ~3) * 4 + (size_t)k * 8 + (size_t)std::min(kprime, kSeedScan) * 8;
   PANO_CUDA(cudaFuncSetAttribute(refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)std::max<size_t>(smem, 48 * 1024)));
   refine_kernel<<<(unsigned)nq, RT, smem, st>>>(a);
