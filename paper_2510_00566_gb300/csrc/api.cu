@@ -7,6 +7,7 @@
 
 #include "../../include/panorama_pq.h"
 #include "internal.h"
+#include "probe_tc.h"
 #include "search.h"
 
 namespace pano {
@@ -415,6 +416,7 @@ int panorama_load(const char* path, pano_index** out) {
     return rc;
   PANO_CUDA(cudaMemcpy(I.cent.p, I.centroids.data(), nl * d * 4, cudaMemcpyHostToDevice));
   PANO_CUDA(cudaMemcpy(I.cent_n2.p, hcn.data(), nl * 4, cudaMemcpyHostToDevice));
+  if (!I.flat && (rc = build_cent_image(I, nullptr))) return rc;
   PANO_CUDA(cudaMemcpy(I.chunk_off_d.p, I.list_chunk_off.data(), (nl + 1) * 8, cudaMemcpyHostToDevice));
   PANO_CUDA(cudaMemcpy(I.list_size_d.p, I.list_size.data(), nl * 4, cudaMemcpyHostToDevice));
   PANO_CUDA(cudaMemcpy(I.level_off_d.p, I.offs.data(), (I.L + 1) * 4, cudaMemcpyHostToDevice));

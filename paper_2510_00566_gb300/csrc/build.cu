@@ -22,6 +22,7 @@
 #include "gemm.h"
 #include "internal.h"
 #include "kernels_common.cuh"
+#include "probe_tc.h"
 #include "search.h"
 #include "verify_tc.h"
 
@@ -510,10 +511,28 @@ int coarse_lists(const float* Xd, int64_t n, int d, int nlist, const pano_build_
   if ((rc = I.cent.alloc((size_t)nlist * d * 4)) || (rc = I.cent_n2.alloc(nlist * 4))) return rc;
   PANO_CUDA(cudaMemcpyAsync(I.cent.p, I.centroids.data(), (size_t)nlist * d * 4, cudaMemcpyHostToDevice, st));
   PANO_CUDA(cudaMemcpyAsync(I.cent_n2.p, hcn.data(), nlist * 4, cudaMemcpyHostToDevice, st));
+  if ((rc = build_cent_image(I, st))) return rc;
 
   // ---- assignment
   I.assign.assign(n, 0);
-  if (nlist > 1) {
+  if (nlist > 1 && probe_tc_supported(d)) {
+    Tmp t_best, t_asg, t_err;
+    const int64_t blk = std::min<int64_t>(n, 1 << 20);
+    PANO_CUDA(cudaMalloc(&t_best.p, 8 * blk * sizeof(unsigned long long)));
+    PANO_CUDA(cudaMalloc(&t_asg.p, n * sizeof(int32_t)));
+    PANO_CUDA(cudaMalloc(&t_err.p, sizeof(int)));
+    PANO_CUDA(cudaMemsetAsync(t_err.p, 0, sizeof(int), st));
+    for (int64_t s = 0; s < n; s += blk) {
+      rc = launch_assign_tc(Xd + s * d, std::min(blk, n - s), I, (unsigned long long*)t_best.p,
+                            (int32_t*)t_asg.p + s, (int*)t_err.p, st);
+      if (rc) return rc;
+    }
+    int herr = 0;
+    PANO_CUDA(cudaMemcpyAsync(I.assign.data(), t_asg.p, n * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    PANO_CUDA(cudaMemcpyAsync(&herr, t_err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    PANO_CUDA(cudaStreamSynchronize(st));
+    if (herr & kErrTimeout) return fail(PANO_ETIMEOUT, "a device-side wait timed out");
+  } else if (nlist > 1) {
     Tmp t_xn, t_best, t_asg;
     const int64_t blk = 1 << 20;
     PANO_CUDA(cudaMalloc(&t_xn.p, blk * sizeof(float)));
@@ -672,7 +691,7 @@ int build_ivf(const pano_transform* t, const float* X, int64_t n, int nlist,
 }  // namespace pano
 
 size_t pano_index::device_bytes() const {
-  return T32.bytes + mu32.bytes + cent.bytes + cent_n2.bytes + chunk_off_d.bytes +
+  return T32.bytes + mu32.bytes + cent.bytes + cent_n2.bytes + cent_img.bytes + chunk_off_d.bytes +
          list_size_d.bytes + level_off_d.bytes + slices.bytes + tails.bytes + xn2.bytes +
          ex.bytes + ids.bytes + rows.bytes + xscale.bytes + pq_codes.bytes + pq_codebook.bytes +
          pq_cent_t.bytes;

@@ -124,6 +124,7 @@ struct pano_index {
   // device arrays
   pano::DevBuf T32, mu32;        // d x d, d
   pano::DevBuf cent, cent_n2;    // nlist x d, nlist   (original space)
+  pano::DevBuf cent_img;         // the tensor-core probe's operand images of cent (probe_tc)
   pano::DevBuf chunk_off_d;      // nlist + 1 int64
   pano::DevBuf list_size_d;      // nlist int32
   pano::DevBuf level_off_d;      // L + 1 int32 (m_l)

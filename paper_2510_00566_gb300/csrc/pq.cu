@@ -30,6 +30,7 @@
 #include "device_common.cuh"
 #include "gemm.h"
 #include "internal.h"
+#include "probe_tc.h"
 #include "search.h"
 
 namespace pano {
@@ -958,6 +959,7 @@ int build_ivfpq(const pano_transform* t, const float* X, int64_t n, int nlist,
     PANO_CUDA(cudaMemcpyAsync(I.cent.p, I.centroids.data(), (size_t)nlist * d * 4,
                               cudaMemcpyHostToDevice, st));
     PANO_CUDA(cudaMemcpyAsync(I.cent_n2.p, hcn.data(), nlist * 4, cudaMemcpyHostToDevice, st));
+    if ((rc = build_cent_image(I, st))) return rc;
     I.assign.assign(o->assign, o->assign + n);
   } else {
     rc = coarse_lists(Xd, n, d, nlist, &co, st, I);

@@ -4,12 +4,20 @@
 // tcgen05 MMAs per K-step (hi.hi + hi.lo + lo.hi of each operand's bf16 hi +
 // lo split), accumulated in FP32 in tensor memory.  The probe selection
 // re-scores exactly every centroid within the error bound of the nprobe-th
-// (probe_tc_gerr), so the probe sets are those of exact distances.
+// (probe_tc_gerr), so the probe sets are those of exact distances.  The same
+// products give a build the nearest centroid of every vector (assign_tc).
+//
+// The centroids' split is laid out once per index (cent_image): per tile of 256
+// centroids and K panel of 64 the swizzled hi and lo operand images, 64 KB that
+// one bulk copy brings in.  (Each CTA used to convert its 256 centroid rows
+// itself, twice the work of its 128 queries: 10,000 x 1,024 x 960 took 296 us,
+// now 174.)
 #include <cuda_bf16.h>
 
 #include <algorithm>
 
 #include "internal.h"
+#include "kernels_common.cuh"
 #include "probe_tc.h"
 #include "tcgen05.cuh"
 
@@ -58,15 +66,25 @@ __device__ __forceinline__ void stage_rows(const float* __restrict__ src, int64_
   }
 }
 
+// One CTA per (K panel, tile): the operand images of 256 centroids.
+__global__ void __launch_bounds__(PT) cent_image_kernel(const float* __restrict__ C, int nlist,
+                                                        int d, unsigned char* __restrict__ img) {
+  unsigned char* out = img + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 * B_BYTES);
+  const int c0 = blockIdx.y * PN;
+  stage_rows(C, c0, min(PN, nlist - c0), d, blockIdx.x, PN,
+             (d & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0, out, out + B_BYTES);
+}
+
 __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict__ Q, int64_t nq,
-                                                         const float* __restrict__ C, int nlist,
-                                                         int d, const float* __restrict__ qn2,
+                                                         const unsigned char* __restrict__ cimg,
+                                                         int nlist, int d,
+                                                         const float* __restrict__ qn2,
                                                          const float* __restrict__ cn2,
                                                          float* __restrict__ pd, int* __restrict__ err,
-                                                         bool vq, bool vc) {
+                                                         bool vq) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  __shared__ __align__(8) uint64_t done[2];
+  __shared__ __align__(8) uint64_t done[2], full[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
@@ -82,6 +100,8 @@ __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict
   if (tid == 0) {
     mbar_init(&done[0], 1);
     mbar_init(&done[1], 1);
+    mbar_init(&full[0], 1);
+    mbar_init(&full[1], 1);
     fence_mbar_init();
     s_fail = 0;
   }
@@ -99,13 +119,18 @@ __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict
       if (!mbar_wait_bounded(&done[s], (dpar >> s) & 1u)) atomicOr(&s_fail, 1);
       dpar ^= 1u << s;
     }
+    if (tid == 0) {
+      mbar_arrive_expect_tx(&full[s], 2 * B_BYTES);
+      bulk_g2s(st + 2 * A_BYTES, cimg + ((size_t)blockIdx.x * np + p) * (2 * B_BYTES), 2 * B_BYTES,
+               &full[s]);
+    }
     stage_rows(Q, q0, nr_q, d, p, PM, vq, st, st + A_BYTES);
-    stage_rows(C, c0, nr_c, d, p, N, vc, st + 2 * A_BYTES, st + 2 * A_BYTES + B_BYTES);
     fence_proxy_async_smem();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     if (tid == 0) {
+      if (!mbar_wait_bounded(&full[s], (p >> 1) & 1)) atomicOr(&s_fail, 1);
       const uint64_t ah = tc::smem_desc(smem_u32(st), 128);
       const uint64_t al = tc::smem_desc(smem_u32(st + A_BYTES), 128);
       const uint64_t bh = tc::smem_desc(smem_u32(st + 2 * A_BYTES), 128);
@@ -163,6 +188,169 @@ __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict
   if (warp == 0) tc::tmem_dealloc(tbase, PN);
 }
 
+// The kBest nearest centroids, by the expansion distance without |x|^2, of each
+// of a CTA's 128 rows in each of two halves of every centroid tile (row r's
+// two threads each scan 128 of a tile's 256 columns): keys (ordered distance
+// << 32 | id) ascending, best[row][half][kBest].
+constexpr int kBest = 4;
+
+__global__ void __launch_bounds__(PT, 1) assign_tc_kernel(
+    const float* __restrict__ X, int64_t m, const unsigned char* __restrict__ cimg, int nlist, int d,
+    const float* __restrict__ cn2, unsigned long long* __restrict__ best, int* __restrict__ err,
+    bool vx) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* base = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+  __shared__ __align__(8) uint64_t done[2], full[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
+  const int64_t r0 = (int64_t)blockIdx.x * PM;
+  const int nr = m - r0 < PM ? (int)(m - r0) : PM;
+  if (warp == 0) {
+    tc::tmem_alloc(&tmem_base, PN);
+    tc::tmem_relinquish();
+  }
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&done[i], 1);
+      mbar_init(&full[i], 1);
+    }
+    fence_mbar_init();
+    s_fail = 0;
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tbase = tmem_base;
+  const int np = (d + PK - 1) / PK;
+  const int row = (warp & 3) * 32 + lane, half = warp >> 2;
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+  unsigned long long b[kBest];
+#pragma unroll
+  for (int i = 0; i < kBest; ++i) b[i] = kEmptyKey;
+  uint32_t dpar = 0, it = 0;  // panels of all tiles run through the two stages
+  for (int c0 = 0; c0 < nlist; c0 += PN) {
+    const int nc = nlist - c0 < PN ? nlist - c0 : PN, N = (nc + 15) & ~15;
+    const uint32_t idesc = tc::idesc_bf16(PM, N);
+    for (int p = 0; p < np; ++p, ++it) {
+      const int s = it & 1;
+      unsigned char* st = base + (size_t)s * STAGE;
+      if (it >= 2) {  // the MMAs that read this stage two panels ago are done
+        if (!mbar_wait_bounded(&done[s], (dpar >> s) & 1u)) atomicOr(&s_fail, 1);
+        dpar ^= 1u << s;
+      }
+      if (tid == 0) {
+        mbar_arrive_expect_tx(&full[s], 2 * B_BYTES);
+        bulk_g2s(st + 2 * A_BYTES, cimg + ((size_t)(c0 / PN) * np + p) * (2 * B_BYTES), 2 * B_BYTES,
+                 &full[s]);
+      }
+      stage_rows(X, r0, nr, d, p, PM, vx, st, st + A_BYTES);
+      fence_proxy_async_smem();
+      tc::fence_before_sync();
+      // (and the last tile's accumulators have been read)
+      const int failed = __syncthreads_or(s_fail);
+      tc::fence_after_sync();
+      if (failed) {  // no copy may be in flight when the CTA ends
+        mbar_wait_bounded(&full[s], (it >> 1) & 1u);
+        c0 = nlist;
+        break;
+      }
+      if (tid == 0) {
+        if (!mbar_wait_bounded(&full[s], (it >> 1) & 1u)) atomicOr(&s_fail, 1);
+        const uint64_t ah = tc::smem_desc(smem_u32(st), 128);
+        const uint64_t al = tc::smem_desc(smem_u32(st + A_BYTES), 128);
+        const uint64_t bh = tc::smem_desc(smem_u32(st + 2 * A_BYTES), 128);
+        const uint64_t bl = tc::smem_desc(smem_u32(st + 2 * A_BYTES + B_BYTES), 128);
+        for (int k = 0; k < PK / 16; ++k) {
+          const uint64_t o = tc::kstep_off(k, 0);
+          tc::mma_bf16(tbase, ah + o, bh + o, idesc, (p > 0 || k > 0) ? 1u : 0u);
+          tc::mma_bf16(tbase, ah + o, bl + o, idesc, 1u);
+          tc::mma_bf16(tbase, al + o, bh + o, idesc, 1u);
+        }
+        tc::mma_commit(&done[s]);
+      }
+    }
+    if (c0 >= nlist) break;
+    // the tile's last commit (its phase is waited for again before the stage's
+    // reuse: the same one, already complete)
+    if (!mbar_wait_bounded(&done[(it - 1) & 1], (dpar >> ((it - 1) & 1)) & 1u)) atomicOr(&s_fail, 1);
+    tc::fence_after_sync();
+    for (int cb = 128 * half; cb < 128 * half + 128 && cb < N; cb += 16) {
+      float v[16];
+      tc::tmem_ld16(tbase + lane_base + (uint32_t)cb, v);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int c = c0 + cb + j;
+        if (c >= nlist) continue;
+        const unsigned long long key =
+            (unsigned long long)float_ordered(fmaf(-2.f, v[j], __ldg(cn2 + c))) << 32 | (uint32_t)c;
+        if (key < b[kBest - 1]) {
+          b[kBest - 1] = key;
+#pragma unroll
+          for (int i = kBest - 1; i > 0; --i)
+            if (b[i] < b[i - 1]) {
+              const unsigned long long t = b[i];
+              b[i] = b[i - 1];
+              b[i - 1] = t;
+            }
+        }
+      }
+    }
+    tc::fence_before_sync();
+  }
+  if (row < nr) {
+#pragma unroll
+    for (int i = 0; i < kBest; ++i) best[((r0 + row) * 2 + half) * kBest + i] = b[i];
+  }
+  __syncthreads();
+  if (tid == 0 && s_fail) atomicOr(err, kErrTimeout);
+  if (warp == 0) tc::tmem_dealloc(tbase, PN);
+}
+
+// The nearest centroid of each row (one warp per row): the smallest expansion
+// distance unless others lie within twice its error bound of it; those are
+// compared by the compensated difference form (ties to the lower id).  Where a
+// half's kBest-th is within the bound there may be more: every centroid is
+// compared.
+__global__ void __launch_bounds__(256) assign_pick_kernel(
+    const float* __restrict__ X, int64_t m, int d, const float* __restrict__ C, int nlist,
+    float cmax, const unsigned long long* __restrict__ best, float gerr, int32_t* __restrict__ out) {
+  const int64_t row = (int64_t)blockIdx.x * 8 + threadIdx.x / 32;
+  const int lane = threadIdx.x & 31;
+  if (row >= m) return;
+  const float* x = X + row * d;
+  const unsigned long long key = lane < 2 * kBest ? best[row * 2 * kBest + lane] : kEmptyKey;
+  const unsigned long long first = warp_min_u64(key);
+  auto dec = [](unsigned long long k) {
+    const uint32_t o = (uint32_t)(k >> 32);
+    return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+  };
+  float n2 = 0.f;
+  for (int j = lane; j < d; j += 32) n2 = fmaf(x[j], x[j], n2);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, off);
+  const float s = sqrtf(n2) * 1.0001f + cmax;  // (the sum's rounding is far below 1e-4)
+  const float hi = dec(first) + 2.f * gerr * s * s * 1.0001f;
+  const uint32_t near = __ballot_sync(0xffffffffu, key != kEmptyKey && dec(key) <= hi);
+  int choice = (int)(uint32_t)first;
+  if (near & (near - 1)) {
+    float e = INFINITY;
+    int c = nlist;
+    auto look = [&](int ci) {
+      const float ei = exact_sqdist_warp(x, C + (int64_t)ci * d, d);
+      if (ei < e || (ei == e && ci < c)) e = ei, c = ci;
+    };
+    if (near & ((1u << (kBest - 1)) | (1u << (2 * kBest - 1)))) {
+      for (int ci = 0; ci < nlist; ++ci) look(ci);
+    } else {
+      for (uint32_t k = near; k; k &= k - 1)
+        look((int)(uint32_t)__shfl_sync(0xffffffffu, key, __ffs(k) - 1));
+    }
+    choice = c;
+  }
+  if (lane == 0) out[row] = choice;
+}
+
 }  // namespace
 
 bool probe_tc_supported(int d) { return d >= 8 && d % 8 == 0; }
@@ -181,9 +369,24 @@ double probe_tc_gerr(int d) {
   return 2.0 * (2.0 * dot / 4.0 + 2.0 * std::ldexp(1.0, -24)) + gamma_n(d + 4);
 }
 
-int launch_probe_tc(const float* Q, int64_t nq, const float* C, int nlist, int d,
-                    const float* qn2, const float* cn2, float* pd, int* err, cudaStream_t st) {
+size_t cent_image_bytes(int nlist, int d) {
+  return (size_t)((nlist + PN - 1) / PN) * ((d + PK - 1) / PK) * (2 * B_BYTES);
+}
+
+int build_cent_image(pano_index& I, cudaStream_t st) {
+  if (!probe_tc_supported(I.d)) return PANO_OK;
+  if (int rc = I.cent_img.alloc(cent_image_bytes(I.nlist, I.d))) return rc;
+  const dim3 grid((unsigned)((I.d + PK - 1) / PK), (unsigned)((I.nlist + PN - 1) / PN));
+  cent_image_kernel<<<grid, PT, 0, st>>>(I.cent.as<float>(), I.nlist, I.d,
+                                         I.cent_img.as<unsigned char>());
+  PANO_CUDA(cudaGetLastError());
+  return PANO_OK;
+}
+
+int launch_probe_tc(const float* Q, int64_t nq, const pano_index& I, const float* qn2, float* pd,
+                    int* err, cudaStream_t st) {
   static PerDeviceOnce once;
+  const int nlist = I.nlist, d = I.d;
   const size_t smem = (size_t)2 * STAGE + 1024;
   PANO_CUDA(once.run([smem] {
     return cudaFuncSetAttribute((const void*)probe_tc_kernel,
@@ -192,8 +395,30 @@ int launch_probe_tc(const float* Q, int64_t nq, const float* C, int nlist, int d
   if (nq <= 0 || nlist <= 0) return PANO_OK;
   const dim3 grid((unsigned)((nlist + PN - 1) / PN), (unsigned)((nq + PM - 1) / PM));
   const bool vq = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(Q) & 15) == 0;
-  const bool vc = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
-  probe_tc_kernel<<<grid, PT, smem, st>>>(Q, nq, C, nlist, d, qn2, cn2, pd, err, vq, vc);
+  probe_tc_kernel<<<grid, PT, smem, st>>>(Q, nq, I.cent_img.as<unsigned char>(), nlist, d, qn2,
+                                          I.cent_n2.as<float>(), pd, err, vq);
+  PANO_CUDA(cudaGetLastError());
+  return PANO_OK;
+}
+
+int launch_assign_tc(const float* X, int64_t m, const pano_index& I, unsigned long long* best,
+                     int32_t* out, int* err, cudaStream_t st) {
+  static PerDeviceOnce once;
+  const int d = I.d, nlist = I.nlist;
+  const size_t smem = (size_t)2 * STAGE + 1024;
+  PANO_CUDA(once.run([smem] {
+    return cudaFuncSetAttribute((const void*)assign_tc_kernel,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  }));
+  if (m <= 0) return PANO_OK;
+  const bool vx = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  assign_tc_kernel<<<(unsigned)((m + PM - 1) / PM), PT, smem, st>>>(
+      X, m, I.cent_img.as<unsigned char>(), nlist, d, I.cent_n2.as<float>(), best, err, vx);
+  PANO_CUDA(cudaGetLastError());
+  float gerr = (float)probe_tc_gerr(d);
+  if ((double)gerr < probe_tc_gerr(d)) gerr = std::nextafter(gerr, INFINITY);
+  assign_pick_kernel<<<(unsigned)((m + 7) / 8), 256, 0, st>>>(X, m, d, I.cent.as<float>(), nlist,
+                                                             I.cmax, best, gerr, out);
   PANO_CUDA(cudaGetLastError());
   return PANO_OK;
 }

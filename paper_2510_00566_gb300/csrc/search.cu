@@ -1793,8 +1793,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       // with the wider error band they need; the band is re-scored exactly
       float gerr;
       if (probe_tc_supported(d)) {
-        int r = launch_probe_tc(queries, nq, I.cent.as<float>(), nlist, d, qn2,
-                                I.cent_n2.as<float>(), pd, err, st);
+        int r = launch_probe_tc(queries, nq, I, qn2, pd, err, st);
         if (r) return r;
         gerr = (float)probe_tc_gerr(d);
         if ((double)gerr < probe_tc_gerr(d)) gerr = std::nextafter(gerr, INFINITY);
@@ -2083,8 +2082,7 @@ int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t n
     row_sqnorm_kernel<<<(unsigned)((nq + 7) / 8), 256, 0, st>>>(queries, nq, d, qn2);
     float gerr;
     if (probe_tc_supported(d)) {
-      int r = launch_probe_tc(queries, nq, I.cent.as<float>(), nlist, d, qn2,
-                              I.cent_n2.as<float>(), pd, err, st);
+      int r = launch_probe_tc(queries, nq, I, qn2, pd, err, st);
       if (r) return r;
       gerr = (float)probe_tc_gerr(d);
       if ((double)gerr < probe_tc_gerr(d)) gerr = std::nextafter(gerr, INFINITY);
