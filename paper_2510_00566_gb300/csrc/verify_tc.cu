@@ -90,34 +90,34 @@ __global__ void __launch_bounds__(256) pack_bf16_kernel(
     const int64_t slot = g * CH + i;
     const bool valid = pb[i] >= 0;
     const float* x = xblk + (int64_t)i * d;
-    double suffix = 0.0, qerr = 0.0;
+    RowBounds rb;
+    Acc2 qerr{0.f, 0.f};
     for (int l = L - 1; l >= 0; --l) {
-      double e = 0.0;
+      Acc2 e{0.f, 0.f};
       if (valid)
         for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) {
-          double xf = x[j];
-          double xh = __bfloat162float(__float2bfloat16_rn(x[j]));
-          e += xh * xh;
-          qerr += (xh - xf) * (xh - xf);
+          const float xf = x[j], xh = __bfloat162float(__float2bfloat16_rn(xf));
+          acc2_sq(e, xh);
+          acc2_sq(qerr, __fsub_rn(xh, xf));  // (exact: xh is within a factor 2 of xf)
         }
-      suffix += warp_sum_f64(e);
-      if (lane == 0)
-        tails[(g * (L + 1) + l) * CH + i] = __double2float_ru(sqrt(suffix * (1.0 + 1e-12)));
+      rb.level(l, e);
     }
-    qerr = warp_sum_f64(qerr);
-    double dev = 0.0;
+    Acc2 dev{0.f, 0.f};
     if (valid) {
       const float* r = rows + (lc * CH + i) * (int64_t)d;
-      for (int j = lane; j < d; j += 32) {
-        double v = (double)r[j] - (double)mu[j];
-        dev += v * v;
-      }
+      for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
     }
-    dev = warp_sum_f64(dev);
+    // lanes 0 and 1 take a root each (FP64 roots are long)
+    const double qe = acc2_f64(warp_sum_acc2(qerr)), de = acc2_f64(warp_sum_acc2(dev));
+    const double root = sqrt(lane == 0 ? qe : de);
+    const double dev_root = __shfl_sync(0xffffffffu, root, 1);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail_norm(u);
     if (lane == 0) {
       tails[(g * (L + 1) + L) * CH + i] = 0.f;
-      xn2[slot] = (float)suffix;
-      ex[slot] = valid ? __double2float_ru((sqrt(qerr) + c_trans * sqrt(dev)) * (1.0 + 1e-9)) : 0.f;
+      xn2[slot] = (float)rb.energy;
+      ex[slot] = valid ? __double2float_ru((root + c_trans * dev_root) * (1.0 + 2e-9)) : 0.f;
       ids[slot] = valid ? (int32_t)pb[i] : -1;
     }
   }
@@ -181,34 +181,34 @@ __global__ void __launch_bounds__(256) pack_fp8_kernel(
     const bool valid = pb[i] >= 0;
     const float* x = xblk + (int64_t)i * d;
     const float sc = s_scale[i], inv = s_inv[i];
-    double suffix = 0.0, qerr = 0.0;
+    RowBounds rb;
+    Acc2 qerr{0.f, 0.f};
     for (int l = L - 1; l >= 0; --l) {
-      double e = 0.0;
+      Acc2 e{0.f, 0.f};
       if (valid)
         for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) {
-          const double xf = x[j];
-          const double xh = (double)(tc::e4m3_to_f32(tc::f32_to_e4m3(x[j] * inv)) * sc);
-          e += xh * xh;
-          qerr += (xh - xf) * (xh - xf);
+          const float xf = x[j], xh = tc::e4m3_to_f32(tc::f32_to_e4m3(xf * inv)) * sc;
+          acc2_sq(e, xh);
+          acc2_sqdiff(qerr, xh, xf);
         }
-      suffix += warp_sum_f64(e);
-      if (lane == 0)
-        tails[(g * (L + 1) + l) * CH + i] = __double2float_ru(sqrt(suffix * (1.0 + 1e-12)));
+      rb.level(l, e);
     }
-    qerr = warp_sum_f64(qerr);
-    double dev = 0.0;
+    Acc2 dev{0.f, 0.f};
     if (valid) {
       const float* r = rows + (lc * CH + i) * (int64_t)d;
-      for (int j = lane; j < d; j += 32) {
-        double v = (double)r[j] - (double)mu[j];
-        dev += v * v;
-      }
+      for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
     }
-    dev = warp_sum_f64(dev);
+    // lanes 0 and 1 take a root each (FP64 roots are long)
+    const double qe = acc2_f64(warp_sum_acc2(qerr)), de = acc2_f64(warp_sum_acc2(dev));
+    const double root = sqrt(lane == 0 ? qe : de);
+    const double dev_root = __shfl_sync(0xffffffffu, root, 1);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail_norm(u);
     if (lane == 0) {
       tails[(g * (L + 1) + L) * CH + i] = 0.f;
-      xn2[slot] = (float)suffix;
-      ex[slot] = valid ? __double2float_ru((sqrt(qerr) + c_trans * sqrt(dev)) * (1.0 + 1e-9)) : 0.f;
+      xn2[slot] = (float)rb.energy;
+      ex[slot] = valid ? __double2float_ru((root + c_trans * dev_root) * (1.0 + 2e-9)) : 0.f;
       xscale[slot] = sc;
       ids[slot] = valid ? (int32_t)pb[i] : -1;
     }
