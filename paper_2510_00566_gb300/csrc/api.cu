@@ -339,6 +339,7 @@ int panorama_load(const char* path, pano_index** out) {
   auto idx = std::make_unique<pano_index>();
   pano_index& I = *idx;
   I.device = dev;
+  if ((rc = I.ws.create(dev))) return rc;
   r.pod(I.n);
   r.pod(I.d);
   r.pod(I.nlist);

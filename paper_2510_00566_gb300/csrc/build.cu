@@ -423,6 +423,27 @@ int DevBuf::alloc(size_t n) {
   return PANO_OK;
 }
 
+int WsPool::create(int device) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = device;
+  PANO_CUDA(cudaMemPoolCreate(&pool, &props));
+  uint64_t keep = kKeep;
+  int off = 0;
+  PANO_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  PANO_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off));
+  return PANO_OK;
+}
+
+cudaError_t WsPool::alloc(void** p, size_t bytes, cudaStream_t st) const {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return e;
+  if (cap != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
 void DevBuf::release() {
   if (p) cudaFree(p);
   p = nullptr;
@@ -568,6 +589,7 @@ int build_ivf(const pano_transform* t, const float* X, int64_t n, int nlist,
   auto idx = std::make_unique<pano_index>();
   pano_index& I = *idx;
   I.device = dev;
+  if ((rc = I.ws.create(dev))) return rc;
   I.n = n;
   I.d = d;
   I.nlist = nlist;

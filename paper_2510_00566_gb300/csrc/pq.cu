@@ -912,6 +912,7 @@ int build_ivfpq(const pano_transform* t, const float* X, int64_t n, int nlist,
   auto idx = std::make_unique<pano_index>();
   pano_index& I = *idx;
   I.device = dev;
+  if ((rc = I.ws.create(dev))) return rc;
   I.n = n;
   I.d = d;
   I.nlist = nlist;
@@ -1172,7 +1173,7 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
   const size_t o_kq = take((size_t)nq * 4);
   const size_t o_stats = take(16 * 8);
   void* ws = nullptr;
-  PANO_CUDA(cudaMallocAsync(&ws, off, st));
+  PANO_CUDA(I.ws.alloc(&ws, off, st));
   char* W = (char*)ws;
   float* qt = (float*)(W + o_qt);
   int32_t* probes = (int32_t*)(W + o_pr);
@@ -1204,7 +1205,7 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     PANO_CUDA(gemm_nt(kStore, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(),
                       d, qt, d, nullptr, nullptr, st));
     mark(1);
-    int rc = probe_only(ip, queries, nq, nprobe, probes, st);
+    int rc = probe_only(ip, queries, nq, nprobe, probes, st, false);
     if (rc) return rc;
     mark(2);
     const unsigned pg = (unsigned)((npairs + 255) / 256);

@@ -368,6 +368,7 @@ int build_flat(const pano_transform* t, const float* X, int64_t n, const pano_bu
   auto idx = std::make_unique<pano_index>();
   pano_index& I = *idx;
   I.device = dev;
+  if ((rc = I.ws.create(dev))) return rc;
   I.n = n;
   I.d = d;
   I.nlist = 1;
@@ -451,7 +452,7 @@ int refine(const pano_index* ip, const float* queries, int64_t nq, const int64_t
   const size_t total = o_err + 256;
   Buf ws;
   ws.st = st;
-  PANO_CUDA(cudaMallocAsync(&ws.p, total, st));
+  PANO_CUDA(I.ws.alloc(&ws.p, total, st));
   char* W = (char*)ws.p;
   PANO_CUDA(cudaMemsetAsync(W + o_err, 0, 256, st));
   int rc = transform_queries(I, queries, nq, (float*)(W + o_qt), (float4*)(W + o_qi),

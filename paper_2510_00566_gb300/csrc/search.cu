@@ -15,6 +15,7 @@
 //   a10 top-k              lock-free k-smallest insertion per query; its k-th
 //                          key is the running threshold d_k      [Alg. 1]
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -326,57 +327,85 @@ __global__ void inv_count_kernel(int64_t nq, const int32_t* __restrict__ probes,
   atomicAdd(&cnt[(r < first_rank_b ? 0 : nlist) + c], 1);
 }
 
+// Exclusive sums over the block's threads of three values each (1024 threads);
+// the totals come back in tot[0..2].
+__device__ __forceinline__ void block_scan3(int (&v)[3], int (&tot)[3]) {
+  __shared__ int part[3][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+  int inc[3];
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    inc[u] = v[u];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, inc[u], off);
+      if (lane >= off) inc[u] += y;
+    }
+    if (lane == 31) part[u][warp] = inc[u];
+  }
+  __syncthreads();
+  if (warp < 3) {
+    int x = part[warp][lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, off);
+      if (lane >= off) x += y;
+    }
+    part[warp][lane] = x;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    v[u] = inc[u] - v[u] + (warp ? part[u][warp - 1] : 0);
+    tot[u] = part[u][31];
+  }
+  __syncthreads();
+}
+
 // Single CTA: exclusive scans of bucket sizes and of work items per list for
-// both phases.  items(c) = ceil(cnt / QB_phase) * nseg(c).
+// both phases, items(c) = ceil(cnt / QB_phase) * nseg(c), and of phase A's seed
+// groups, ceil(cnt / seed_sub) (soff: nlist entries; null with one list).
+// totals: [2 ph] bucket entries, [2 ph + 1] items, [6] seed groups.  (The 1,024
+// partial sums are scanned by shuffles; one thread adding them up was 20 of the
+// kernel's 26 us, a tenth of a one-query search.)
 __global__ void __launch_bounds__(1024) inv_scan_kernel(const int* __restrict__ cnt, int nlist,
                                                         const int64_t* __restrict__ chunk_off,
-                                                        int seg, int qbA, int qbB,
+                                                        int seg, int qbA, int qbB, int seed_sub,
                                                         int* __restrict__ boff,
                                                         int* __restrict__ ioff,
+                                                        int* __restrict__ soff,
                                                         int* __restrict__ totals) {
-  __shared__ int part_b[1024], part_i[1024];
   for (int ph = 0; ph < 2; ++ph) {
     const int* cn = cnt + ph * nlist;
     const int qb = ph == 0 ? qbA : qbB;
-    int per = (nlist + 1023) / 1024;
-    int b0 = threadIdx.x * per, b1 = min(nlist, b0 + per);
-    int sb = 0, si = 0;
+    const int per = (nlist + 1023) / 1024;
+    const int b0 = min(nlist, (int)threadIdx.x * per), b1 = min(nlist, b0 + per);
+    auto items = [&](int c) {
+      const int nch = (int)(chunk_off[c + 1] - chunk_off[c]);
+      return ((cn[c] + qb - 1) / qb) * ((nch + seg - 1) / seg);
+    };
+    int v[3] = {0, 0, 0}, tot[3];
     for (int c = b0; c < b1; ++c) {
-      int nch = (int)(chunk_off[c + 1] - chunk_off[c]);
-      int nseg = (nch + seg - 1) / seg;
-      sb += cn[c];
-      si += ((cn[c] + qb - 1) / qb) * nseg;
+      v[0] += cn[c];
+      v[1] += items(c);
+      v[2] += (cn[c] + seed_sub - 1) / seed_sub;
     }
-    part_b[threadIdx.x] = sb;
-    part_i[threadIdx.x] = si;
-    __syncthreads();
+    block_scan3(v, tot);
+    for (int c = b0; c < b1; ++c) {
+      boff[ph * (nlist + 1) + c] = v[0];
+      ioff[ph * (nlist + 1) + c] = v[1];
+      if (ph == 0 && soff) soff[c] = v[2];
+      v[0] += cn[c];
+      v[1] += items(c);
+      v[2] += (cn[c] + seed_sub - 1) / seed_sub;
+    }
     if (threadIdx.x == 0) {
-      int ab = 0, ai = 0;
-      for (int t = 0; t < 1024; ++t) {
-        int xb = part_b[t], xi = part_i[t];
-        part_b[t] = ab;
-        part_i[t] = ai;
-        ab += xb;
-        ai += xi;
-      }
-      totals[2 * ph] = ab;
-      totals[2 * ph + 1] = ai;
+      boff[ph * (nlist + 1) + nlist] = tot[0];
+      ioff[ph * (nlist + 1) + nlist] = tot[1];
+      totals[2 * ph] = tot[0];
+      totals[2 * ph + 1] = tot[1];
+      if (ph == 0) totals[6] = tot[2];
     }
-    __syncthreads();
-    int ab = part_b[threadIdx.x], ai = part_i[threadIdx.x];
-    for (int c = b0; c < b1; ++c) {
-      int nch = (int)(chunk_off[c + 1] - chunk_off[c]);
-      int nseg = (nch + seg - 1) / seg;
-      boff[ph * (nlist + 1) + c] = ab;
-      ioff[ph * (nlist + 1) + c] = ai;
-      ab += cn[c];
-      ai += ((cn[c] + qb - 1) / qb) * nseg;
-    }
-    if (threadIdx.x == 1023) {
-      boff[ph * (nlist + 1) + nlist] = ab;
-      ioff[ph * (nlist + 1) + nlist] = ai;
-    }
-    __syncthreads();
   }
 }
 
@@ -397,12 +426,17 @@ __global__ void inv_scatter_kernel(int64_t nq, const int32_t* __restrict__ probe
   bucket[pos] = (int32_t)qi;
 }
 
-// Work item i of a phase -> (list, segment, bucket offset, group size).
-__global__ void inv_emit_kernel(int ph, const int* __restrict__ cnt, int nlist,
-                                const int64_t* __restrict__ chunk_off, int seg, int qb,
+// Work item i of a phase -> (list, segment, bucket offset, group size); phase
+// ph0 + blockIdx.y.
+__global__ void inv_emit_kernel(int ph0, const int* __restrict__ cnt, int nlist,
+                                const int64_t* __restrict__ chunk_off, int seg, int qbA, int qbB,
                                 const int* __restrict__ boff, const int* __restrict__ ioff,
-                                const int* __restrict__ totals, int64_t cap,
-                                int4* __restrict__ items, int* __restrict__ err) {
+                                const int* __restrict__ totals, int64_t capA, int64_t capB,
+                                int4* __restrict__ itA, int4* __restrict__ itB,
+                                int* __restrict__ err) {
+  const int ph = ph0 + blockIdx.y, qb = ph == 0 ? qbA : qbB;
+  const int64_t cap = ph == 0 ? capA : capB;
+  int4* items = ph == 0 ? itA : itB;
   const int n_items = totals[2 * ph + 1];
   const int* io = ioff + ph * (nlist + 1);
   const int* bo = boff + ph * (nlist + 1);
@@ -558,27 +592,34 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
 // and row, each lane sums fl(q_j - x_j)^2 by FMA over its (at most 32) dims
 // into four interleaved sums, then the warp adds the lanes' sums: each term
 // meets at most m = ceil(d/128) + 8 roundings, as in seed_tau_kernel, whose
-// slack is reused.  CTA b takes sub-group b % nsub of item b / nsub; only
-// an item's first segment computes (the queries of a group are the same in
-// every segment).
+// slack is reused.  CTA b takes seed group b: 16 of the queries of one list,
+// found by their scan soff (a CTA per possible work item left nearly all of
+// them without work where one list is long: 1.37 ms for 16,384 queries on
+// Zipf-sized lists).
 constexpr int kSeedSub = 16;
 
 __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
-    const float* __restrict__ q, int d, const int4* __restrict__ items,
-    const int* __restrict__ n_items, int64_t items_cap, int nsub,
+    const float* __restrict__ q, int d, const int* __restrict__ soff, int nlist,
+    const int* __restrict__ totals, const int* __restrict__ cnt, const int* __restrict__ boff,
     const int32_t* __restrict__ bucket, const int64_t* __restrict__ chunk_off,
     const int32_t* __restrict__ list_size, int chunk, const float* __restrict__ rows,
     const int32_t* __restrict__ kq, float slack, float* __restrict__ tau_seed,
     const int32_t* __restrict__ ids, unsigned long long* __restrict__ topk, int k_max) {
   extern __shared__ float4 sg_raw[];
-  const int64_t item = blockIdx.x / nsub;
-  const int sub = blockIdx.x % nsub;
-  if (item >= imin64(*n_items, items_cap)) return;
-  const int4 it = items[item];
-  if (it.y != 0) return;
-  const int g0 = sub * kSeedSub, G = min(kSeedSub, it.w - g0);
+  const int b = (int)blockIdx.x;
+  if (b >= totals[6]) return;
+  int c = 0;
+  if (soff) {  // the last list whose first group is at most b (it has one: b is within the total)
+    int hi = nlist;
+    while (hi - c > 1) {
+      const int mid = (c + hi) >> 1;
+      if (soff[mid] <= b) c = mid;
+      else hi = mid;
+    }
+  }
+  const int g0 = (b - (soff ? soff[c] : 0)) * kSeedSub, G = min(kSeedSub, cnt[c] - g0);
   if (G <= 0) return;
-  const int c = it.x, n = list_size[c];
+  const int n = list_size[c];
   const int d4 = d >> 2;
   float4* qs = sg_raw;                                                // [G][d/4]
   float* dist = reinterpret_cast<float*>(sg_raw + (size_t)kSeedSub * d4);  // [G][kSeedMax]
@@ -586,7 +627,7 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
   __shared__ float s_t[kSeedSub];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
   if (tid < G) {
-    const int qi = bucket[it.z + g0 + tid];
+    const int qi = bucket[boff[c] + g0 + tid];
     const int k = kq[qi];
     s_q[tid] = qi;
     s_k[tid] = k;
@@ -1514,6 +1555,14 @@ cudaError_t allow_dynamic_smem(const void* kern) {
                               optin - (int)fa.sharedSizeBytes);
 }
 
+// Once per kernel and device: the two attribute calls cost a small search more
+// than its launch.
+template <auto* KERN>
+cudaError_t allow_dynamic_smem_once() {
+  static PerDeviceOnce once;
+  return once.run([] { return allow_dynamic_smem((const void*)KERN); });
+}
+
 // FP32 verify tiles (QB queries x CB candidates, NTH threads).  Phase A
 // (each query's nearest list: small groups) prefers wide candidate tiles,
 // phase B (many queries per list) 64-query groups; narrower tiles serve wide
@@ -1529,17 +1578,19 @@ constexpr TileCfg kTilesB[] = {{64, 64, 256, 4}, {32, 64, 128, 4}, {16, 64, 64, 
 template <int QB, int CB, int NTH, int NST, bool LARGE>
 cudaError_t tile_kernel_attrs(const void** kern, size_t* static_smem) {
   static PerDeviceOnce once;
+  static std::atomic<size_t> bytes{0};  // (the kernel's, the same on every device)
   auto k = verify_fp32_kernel<QB, CB, NTH, NST, LARGE>;
   cudaError_t err = once.run([&] {
     cudaError_t e = allow_dynamic_smem((const void*)k);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess) bytes = fa.sharedSizeBytes;
     return e;
   });
-  cudaFuncAttributes fa;
-  if (err == cudaSuccess) err = cudaFuncGetAttributes(&fa, k);
   *kern = (const void*)k;
-  *static_smem = err == cudaSuccess ? fa.sharedSizeBytes : 0;
+  *static_smem = err == cudaSuccess ? bytes.load() : 0;
   return err;
 }
 
@@ -1617,6 +1668,7 @@ struct SearchLayout {
   int64_t capA = 0, capB = 0;
   size_t o_qt, o_qinfo, o_qtail, o_qn2, o_pd, o_pr, o_npq, o_kq, o_seed, o_cnt, o_fill, o_boff,
       o_ioff, o_tot, o_bucket, o_itA, o_itB, o_topk, o_err, o_stats;
+  size_t z_bytes = 0;
   size_t total = 0;
 };
 
@@ -1651,17 +1703,20 @@ int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLa
   y.o_npq = cv.take<int32_t>(nq);
   y.o_kq = cv.take<int32_t>(nq);
   y.o_seed = cv.take<float>(nq);
+  // zeroed together: from o_cnt to the end of o_stats; read back together:
+  // from o_tot on
   y.o_cnt = cv.take<int>(2 * (size_t)nlist);
   y.o_fill = cv.take<int>(2 * (size_t)nlist);
+  y.o_tot = cv.take<int>(12);
+  y.o_err = y.o_tot + 8 * sizeof(int);
+  y.o_stats = cv.take<unsigned long long>(kStatWords);
+  y.z_bytes = cv.off - y.o_cnt;
   y.o_boff = cv.take<int>(2 * (size_t)(nlist + 1));
   y.o_ioff = cv.take<int>(2 * (size_t)(nlist + 1));
-  y.o_tot = cv.take<int>(8);
   y.o_bucket = cv.take<int32_t>((size_t)nq * stride);
   y.o_itA = cv.take<int4>(y.capA);
   y.o_itB = cv.take<int4>(std::max<int64_t>(y.capB, 1));
   y.o_topk = cv.take<unsigned long long>((size_t)nq * k_max);
-  y.o_err = cv.take<int>(4);
-  y.o_stats = cv.take<unsigned long long>(kStatWords);
   y.total = cv.off;
   return PANO_OK;
 }
@@ -1727,7 +1782,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
                "search workspace of " + std::to_string(cv.off) + " bytes exceeds the " +
                    std::to_string(ext_cap) + "-byte static scratch");
   } else {
-    PANO_CUDA(cudaMallocAsync(&ws, cv.off, st));
+    PANO_CUDA(I.ws.alloc(&ws, cv.off, st));
   }
   char* W = static_cast<char*>(ws);
   auto P = [&](size_t o) { return (void*)(W + o); };
@@ -1758,12 +1813,8 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     if (timing) cudaEventRecord(ev[i], st);
   };
   auto body = [&]() -> int {
-    PANO_CUDA(cudaMemsetAsync(cnt, 0, 2 * (size_t)nlist * 4, st));
-    PANO_CUDA(cudaMemsetAsync(fillc, 0, 2 * (size_t)nlist * 4, st));
-    PANO_CUDA(cudaMemsetAsync(tot, 0, 8 * 4, st));  // [4..5] verify counters
+    PANO_CUDA(cudaMemsetAsync(cnt, 0, lay.z_bytes, st));  // (tot[4..5]: verify counters)
     PANO_CUDA(cudaMemsetAsync(topk, 0xff, (size_t)nq * k_max * 8, st));
-    PANO_CUDA(cudaMemsetAsync(err, 0, 16, st));
-    PANO_CUDA(cudaMemsetAsync(stats, 0, kStatWords * 8, st));
     prep_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, st>>>(nq, nprobe, nprobe_scalar, np_cap, k,
                                                               k_scalar, k_max, npq, kq, err);
     PANO_CUDA(cudaGetLastError());
@@ -1804,7 +1855,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       }
       const float cmax = I.cmax;
       size_t psm = (size_t)nlist * 4;
-      PANO_CUDA(allow_dynamic_smem((const void*)probe_select_kernel));
+      PANO_CUDA(allow_dynamic_smem_once<probe_select_kernel>());
       probe_select_kernel<<<(unsigned)nq, NT, psm, st>>>(pd, nlist, queries, I.cent.as<float>(), d,
                                                          qn2, cmax, gerr, npq, stride, probes, err,
                                                          0);
@@ -1824,15 +1875,20 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     const int first_rank_b = one_pass ? 0 : 1;
     inv_count_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(nq, probes, stride, npq, cnt,
                                                                    nlist, first_rank_b);
+    // (the seed groups' scan takes the place of the probe distances)
+    int* soff = nlist > 1 ? (int*)P(o_pd) : nullptr;
     inv_scan_kernel<<<1, 1024, 0, st>>>(cnt, nlist, I.chunk_off_d.as<int64_t>(), SEG, QBA, QBB,
-                                        boff, ioff, tot);
+                                        kSeedSub, boff, ioff, soff, tot);
     inv_scatter_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(
         nq, probes, stride, npq, boff, tot, fillc, nlist, first_rank_b, bucket);
     PANO_CUDA(cudaGetLastError());
-    inv_emit_kernel<<<1024, 256, 0, st>>>(0, cnt, nlist, I.chunk_off_d.as<int64_t>(), SEG, QBA,
-                                          boff, ioff, tot, capA, itA, err);
-    inv_emit_kernel<<<1024, 256, 0, st>>>(1, cnt, nlist, I.chunk_off_d.as<int64_t>(), SEG, QBB,
-                                          boff, ioff, tot, capB, itB, err);
+    {
+      const int64_t most = std::max(one_pass ? 0 : capA, capB);
+      const dim3 grid((unsigned)std::min<int64_t>(1024, (most + 255) / 256), one_pass ? 1 : 2);
+      inv_emit_kernel<<<grid, 256, 0, st>>>(one_pass ? 1 : 0, cnt, nlist,
+                                            I.chunk_off_d.as<int64_t>(), SEG, QBA, QBB, boff, ioff,
+                                            tot, capA, capB, itA, itB, err);
+    }
     PANO_CUDA(cudaGetLastError());
     // the warm-start seeds, in phase A's order when there is a phase A (its
     // bucket lists every query once, grouped by nearest list, so the CTAs
@@ -1843,11 +1899,11 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     if ((double)seed_slack < seed_sl) seed_slack = std::nextafter(seed_slack, INFINITY);
     if (!one_pass && d <= 1024 && (d & 3) == 0 &&
         (reinterpret_cast<uintptr_t>(queries) & 15) == 0) {
-      const int nsub = (QBA + kSeedSub - 1) / kSeedSub;
+      const int64_t groups = std::min<int64_t>(nq, (nq + kSeedSub - 1) / kSeedSub + nlist);
       const size_t gsm = (size_t)kSeedSub * d * 4 + (size_t)kSeedSub * kSeedMax * 4;
-      PANO_CUDA(allow_dynamic_smem((const void*)seed_group_kernel));
-      seed_group_kernel<<<(unsigned)(capA * nsub), kSeedWarps * 32, gsm, st>>>(
-          queries, d, itA, tot + 1, capA, nsub, bucket, I.chunk_off_d.as<int64_t>(),
+      PANO_CUDA(allow_dynamic_smem_once<seed_group_kernel>());
+      seed_group_kernel<<<(unsigned)groups, kSeedWarps * 32, gsm, st>>>(
+          queries, d, soff, nlist, tot, cnt, boff, bucket, I.chunk_off_d.as<int64_t>(),
           I.list_size_d.as<int32_t>(), I.chunk, I.rows.as<float>(), kq, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     } else {
@@ -2000,13 +2056,17 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       PANO_CUDA(cudaGetLastError());
     }
     if (sync || collect) {
-      int herr[4];
-      unsigned long long hst[kStatWords];
-      int htot[8];
-      PANO_CUDA(cudaMemcpyAsync(herr, err, 16, cudaMemcpyDeviceToHost, st));
-      PANO_CUDA(cudaMemcpyAsync(hst, stats, kStatWords * 8, cudaMemcpyDeviceToHost, st));
-      PANO_CUDA(cudaMemcpyAsync(htot, tot, 32, cudaMemcpyDeviceToHost, st));
+      // totals, error word and counters in one copy
+      char back[4096];
+      const size_t n_back = lay.o_cnt + lay.z_bytes - o_tot;
+      static_assert(3 * 256 + kStatWords * 8 <= sizeof(back), "the words from o_tot on");
+      PANO_CUDA(cudaMemcpyAsync(back, tot, n_back, cudaMemcpyDeviceToHost, st));
       PANO_CUDA(cudaStreamSynchronize(st));
+      int herr[4], htot[8];
+      unsigned long long hst[kStatWords];
+      std::memcpy(htot, back, sizeof(htot));
+      std::memcpy(herr, back + (o_err - o_tot), sizeof(herr));
+      std::memcpy(hst, back + (o_stats - o_tot), sizeof(hst));
       t_stats.pair_levels = (int64_t)hst[0];
       t_stats.tile_levels = (int64_t)hst[1];
       t_stats.slice_bytes = (int64_t)hst[2];
@@ -2051,7 +2111,7 @@ int status_of_device_error(int word) {
 }
 
 int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t nprobe,
-               int32_t* out, cudaStream_t st) {
+               int32_t* out, cudaStream_t st, bool sync) {
   PANO_CHECK(ip, PANO_EINVAL, "null index");
   const pano_index& I = *ip;
   PANO_CHECK(nprobe >= 1 && nprobe <= I.nlist, PANO_EINVAL, "nprobe must be in [1, nlist]");
@@ -2069,7 +2129,7 @@ int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t n
   size_t o_np = cv.take<int32_t>(2 * nq);
   size_t o_err = cv.take<int>(4);
   void* ws = nullptr;
-  PANO_CUDA(cudaMallocAsync(&ws, cv.off, st));
+  PANO_CUDA(I.ws.alloc(&ws, cv.off, st));
   char* W = (char*)ws;
   float* pd = (float*)(W + o_pd);
   float* qn2 = (float*)(W + o_qn);
@@ -2092,11 +2152,11 @@ int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t n
       gerr = (float)(2.0 * gamma_n(gemm_rounds(d) + 4));
     }
     size_t psm = (size_t)nlist * 4;
-    PANO_CUDA(allow_dynamic_smem((const void*)probe_select_kernel));
+    PANO_CUDA(allow_dynamic_smem_once<probe_select_kernel>());
     probe_select_kernel<<<(unsigned)nq, NT, psm, st>>>(pd, nlist, queries, I.cent.as<float>(), d,
                                                        qn2, I.cmax, gerr, npq, nprobe, out, err, 1);
     PANO_CUDA(cudaGetLastError());
-    PANO_CUDA(cudaStreamSynchronize(st));
+    if (sync) PANO_CUDA(cudaStreamSynchronize(st));
     return PANO_OK;
   };
   int rc = body();

@@ -17,7 +17,7 @@ int search_workspace_bytes(const pano_index* ip, int64_t nq, int32_t stride, int
 // kErrBadInput -> PANO_EINVAL, otherwise PANO_OK).
 int status_of_device_error(int word);
 int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t nprobe,
-               int32_t* out, cudaStream_t st);
+               int32_t* out, cudaStream_t st, bool sync = true);
 const pano_search_stats& last_stats();
 pano_search_stats& stats_slot();  // the calling thread's last-call statistics
 int transform_queries(const pano_index& I, const float* queries, int64_t nq, float* qt,
