@@ -38,7 +38,15 @@ constexpr int CH = 64;
 // [8..15] section cycles, [16..23] their phase-A part, [24] phase-A pairs,
 // [25] live-row bytes (tensor-core path).
 constexpr int kStatWords = 26;
-constexpr int SEG_CHUNKS = 32;  // chunks per work-item segment
+constexpr int SEG_CHUNKS = 32;  // chunks per work-item segment of a large FP32 batch
+// A small batch takes shorter segments, until there are a few items per SM:
+// 100 queries on one list of 20,000 were 70 items on 152 SMs (295 us, now
+// 103).  `items` counts the batch's (query group, full segment) pairs.
+inline int seg_chunks(int64_t items) {
+  int seg = SEG_CHUNKS;
+  while (seg > 4 && items < 608) seg /= 2, items *= 2;
+  return seg;
+}
 constexpr int NT = 256;
 
 __device__ __forceinline__ int64_t imin64(int64_t a, int64_t b) { return a < b ? a : b; }
@@ -467,7 +475,7 @@ __global__ void inv_emit_kernel(int ph0, const int* __restrict__ cnt, int nlist,
 }
 
 // ------------------------------------------------- Alg. 1 warm start (a6)
-// Per query: distances to the first max(4k, 64) (at most 512) members of its
+// Per query: distances to the first max(4k, 64, n / 64) (at most 512) members of its
 // nearest list; the k-th smallest is an upper bound on d_k and seeds the
 // threshold before any tile is verified.  Algorithm 1 also fills its heap
 // with k candidates before pruning anything; that matters once the
@@ -487,6 +495,11 @@ __global__ void inv_emit_kernel(int ph0, const int* __restrict__ cnt, int nlist,
 // (host-computed, rounded up); multiplying by it (rounding up) keeps every
 // seed distance an upper bound on the exact one.
 constexpr int kSeedMax = 512;
+// (a long list's work items run side by side: none finds a threshold that the
+// others have tightened, so the first one has to be better)
+__device__ __forceinline__ int seed_count(int n, int k) {
+  return min(n, min(kSeedMax, max(max(4 * k, 64), n >> 6)));
+}
 constexpr int kSeedWarps = 8;
 
 __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
@@ -502,7 +515,7 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
   const int k = kq[row];
   const int c = probes[row * stride];
   const int n = c >= 0 ? list_size[c] : 0;
-  const int ns = min(n, min(kSeedMax, max(4 * k, 64)));
+  const int ns = seed_count(n, k);
   if (k <= 0 || ns < k) {
     if (threadIdx.x == 0) tau_seed[row] = k <= 0 ? -1.f : INFINITY;
     return;
@@ -597,11 +610,13 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
 // them without work where one list is long: 1.37 ms for 16,384 queries on
 // Zipf-sized lists).
 constexpr int kSeedSub = 16;
+// (fewer queries per group where 16 would leave SMs without one)
+inline int seed_sub_of(int64_t nq) { return nq >= 16 * 304 ? 16 : nq >= 4 * 304 ? 8 : nq >= 304 ? 4 : 2; }
 
 __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
     const float* __restrict__ q, int d, const int* __restrict__ soff, int nlist,
-    const int* __restrict__ totals, const int* __restrict__ cnt, const int* __restrict__ boff,
-    const int32_t* __restrict__ bucket, const int64_t* __restrict__ chunk_off,
+    const int* __restrict__ totals, int sub_q, const int* __restrict__ cnt,
+    const int* __restrict__ boff, const int32_t* __restrict__ bucket, const int64_t* __restrict__ chunk_off,
     const int32_t* __restrict__ list_size, int chunk, const float* __restrict__ rows,
     const int32_t* __restrict__ kq, float slack, float* __restrict__ tau_seed,
     const int32_t* __restrict__ ids, unsigned long long* __restrict__ topk, int k_max) {
@@ -617,12 +632,12 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
       else hi = mid;
     }
   }
-  const int g0 = (b - (soff ? soff[c] : 0)) * kSeedSub, G = min(kSeedSub, cnt[c] - g0);
+  const int g0 = (b - (soff ? soff[c] : 0)) * sub_q, G = min(sub_q, cnt[c] - g0);
   if (G <= 0) return;
   const int n = list_size[c];
   const int d4 = d >> 2;
   float4* qs = sg_raw;                                                // [G][d/4]
-  float* dist = reinterpret_cast<float*>(sg_raw + (size_t)kSeedSub * d4);  // [G][kSeedMax]
+  float* dist = reinterpret_cast<float*>(sg_raw + (size_t)sub_q * d4);  // [G][kSeedMax]
   __shared__ int s_q[kSeedSub], s_k[kSeedSub], s_ns[kSeedSub];
   __shared__ float s_t[kSeedSub];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
@@ -631,7 +646,7 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
     const int k = kq[qi];
     s_q[tid] = qi;
     s_k[tid] = k;
-    s_ns[tid] = min(n, min(kSeedMax, max(4 * k, 64)));
+    s_ns[tid] = seed_count(n, k);
   }
   __syncthreads();
   int nsmax = 0;
@@ -727,7 +742,7 @@ struct VerifyArgs {
   int* err;
   unsigned long long* stats;  // kStatWords counters (layout at kStatWords)
   int64_t items_cap;
-  int d, L, max_w, k_max;
+  int d, L, max_w, k_max, seg;
   float gslack;    // slack factor: |computed - exact| <= gslack (|q~|+|x~|)^2
   float lb_scale;  // (1 - 8u) / (1 + eta): lower bound in T~ space -> original
   float ub_scale;  // (1 + 8u) / (1 - eta): upper bound in T~ space -> original
@@ -1039,8 +1054,8 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
     const int n_items = (int)imin64(*a.n_items, a.items_cap);
     if (item >= n_items || failed) break;
     const int4 it = a.items[item];
-    const int64_t ch0 = a.chunk_off[it.x] + (int64_t)it.y * SEG_CHUNKS;
-    const int64_t ch1 = imin64(a.chunk_off[it.x + 1], ch0 + SEG_CHUNKS);
+    const int64_t ch0 = a.chunk_off[it.x] + (int64_t)it.y * a.seg;
+    const int64_t ch1 = imin64(a.chunk_off[it.x + 1], ch0 + a.seg);
     const int G = it.w;
     fq = 0u;
     fn = 0;
@@ -1664,7 +1679,7 @@ thread_local pano_search_stats t_stats;
 // tiles of the FP32 verify phases, the work-item capacities and the carve.
 struct SearchLayout {
   TileCfg tileA{TC_QG, 0, 0, 0}, tileB{TC_QG, 0, 0, 0};
-  int bpsA = 0, bpsB = 0;
+  int bpsA = 0, bpsB = 0, seg = 0;
   int64_t capA = 0, capB = 0;
   size_t o_qt, o_qinfo, o_qtail, o_qn2, o_pd, o_pr, o_npq, o_kq, o_seed, o_cnt, o_fill, o_boff,
       o_ioff, o_tot, o_bucket, o_itA, o_itB, o_topk, o_err, o_stats;
@@ -1682,7 +1697,12 @@ int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLa
     if (r) return r;
   }
   const int QBA = y.tileA.QB, QBB = y.tileB.QB;
-  const int SEG = tcpath ? TC_SEG : SEG_CHUNKS;
+  // (an FP32 batch has at least a group per QBA queries in phase A, on lists of
+  // the mean size)
+  const int64_t mean_seg = I.n_chunks / ((int64_t)nlist * SEG_CHUNKS) + 1;
+  const int64_t groups = (nq + QBA - 1) / QBA + std::min<int64_t>(nq, nlist - 1);
+  y.seg = tcpath ? TC_SEG : seg_chunks(groups * mean_seg);
+  const int SEG = y.seg;
   // work-item capacity: groups x segments, plus one partial group per list
   int64_t max_seg = 1, tot_seg = 0;
   for (int c = 0; c < nlist; ++c) {
@@ -1767,7 +1787,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
   const TileCfg tileA = lay.tileA, tileB = lay.tileB;
   const int bpsA = lay.bpsA, bpsB = lay.bpsB;
   const int QBA = tileA.QB, QBB = tileB.QB;
-  const int SEG = tcpath ? TC_SEG : SEG_CHUNKS;
+  const int SEG = lay.seg;
   const int64_t capA = lay.capA, capB = lay.capB;
   const size_t o_qt = lay.o_qt, o_qinfo = lay.o_qinfo, o_qtail = lay.o_qtail, o_qn2 = lay.o_qn2,
                o_pd = lay.o_pd, o_pr = lay.o_pr, o_npq = lay.o_npq, o_kq = lay.o_kq,
@@ -1877,8 +1897,9 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
                                                                    nlist, first_rank_b);
     // (the seed groups' scan takes the place of the probe distances)
     int* soff = nlist > 1 ? (int*)P(o_pd) : nullptr;
+    const int seed_sub = seed_sub_of(nq);
     inv_scan_kernel<<<1, 1024, 0, st>>>(cnt, nlist, I.chunk_off_d.as<int64_t>(), SEG, QBA, QBB,
-                                        kSeedSub, boff, ioff, soff, tot);
+                                        seed_sub, boff, ioff, soff, tot);
     inv_scatter_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(
         nq, probes, stride, npq, boff, tot, fillc, nlist, first_rank_b, bucket);
     PANO_CUDA(cudaGetLastError());
@@ -1899,11 +1920,11 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     if ((double)seed_slack < seed_sl) seed_slack = std::nextafter(seed_slack, INFINITY);
     if (!one_pass && d <= 1024 && (d & 3) == 0 &&
         (reinterpret_cast<uintptr_t>(queries) & 15) == 0) {
-      const int64_t groups = std::min<int64_t>(nq, (nq + kSeedSub - 1) / kSeedSub + nlist);
-      const size_t gsm = (size_t)kSeedSub * d * 4 + (size_t)kSeedSub * kSeedMax * 4;
+      const int64_t groups = std::min<int64_t>(nq, (nq + seed_sub - 1) / seed_sub + nlist);
+      const size_t gsm = (size_t)seed_sub * d * 4 + (size_t)seed_sub * kSeedMax * 4;
       PANO_CUDA(allow_dynamic_smem_once<seed_group_kernel>());
       seed_group_kernel<<<(unsigned)groups, kSeedWarps * 32, gsm, st>>>(
-          queries, d, soff, nlist, tot, cnt, boff, bucket, I.chunk_off_d.as<int64_t>(),
+          queries, d, soff, nlist, tot, seed_sub, cnt, boff, bucket, I.chunk_off_d.as<int64_t>(),
           I.list_size_d.as<int32_t>(), I.chunk, I.rows.as<float>(), kq, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     } else {
@@ -2004,6 +2025,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     va.L = L;
     va.max_w = I.max_w;
     va.k_max = k_max;
+    va.seg = SEG;
     va.gslack = (float)(2.0 * gamma_n(I.max_w + L + 8));
     va.lb_scale = (float)((1.0 - 8.0 * kU32) / (1.0 + I.eta));
     {

@@ -293,7 +293,7 @@ struct QTerms {
 struct Shared {
   float Hx[S * CH], rx[S * CH], ex[S * CH];  // candidate terms of the separable test
   uint32_t alive[S][2][CH];                  // per chunk and query half: a word per row
-  QTerms qterm[2];                           // by parity of the tested level
+  QTerms qterm;                              // of the tested level
   float qnq[QG], qrq[QG], qeq[QG], qtau[QG];
   float qs[QG], qun[QG];  // E4M3: the query's scale 2^e, its split's underflow per unit of |x|_2
   int32_t qid[QG], qk[QG], bq[QG];  // bq: the B producer's copy of qid
@@ -943,12 +943,10 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
             const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, kk);
             const float tau = key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f);
             set_query_terms(tid, fminf(tau, __ldcg(a.tau_seed + q)),
-                            a.eps * a.qtail[(int64_t)q * (L + 1) + 1], sh.qterm[0]);
+                            a.eps * a.qtail[(int64_t)q * (L + 1) + 1], sh.qterm);
           } else {
-            for (QTerms& qt : sh.qterm) {
-              qt.E[tid] = qt.G[tid] = qt.S[tid] = 0.f;
-              qt.H[tid] = -INFINITY;
-            }
+            sh.qterm.E[tid] = sh.qterm.G[tid] = sh.qterm.S[tid] = 0.f;
+            sh.qterm.H[tid] = -INFINITY;
             sh.qtau[tid] = -1.f;
           }
         }
@@ -980,7 +978,6 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
       // ---- the tested levels
       ChunkState cs;
       cs.start(nch, first_test);
-      int parity = 0;  // the query-term buffer
       for (int l = first_test, l0 = 0;;) {
         bool ok = true;
         uint32_t test = 0;
@@ -1019,16 +1016,23 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
           return m ? __ldg(tail + (__ffs(m) - 1) * (L + 1) * CH) : 0.f;
         };
         float sx_n = tail_of(test);
-        if (l > 0 && tid < QG && sh.qk[tid] > 0) {  // (level 0's terms: the prologue)
+        // Level 0's terms were set in the prologue.  At a level in between only
+        // the query's tail norm changes: the threshold stays the item's first
+        // one (an older threshold is a larger one: still valid), whose words
+        // and terms were 4k of a tested level's cycles.  The last level takes
+        // the threshold of the moment.
+        if (l > 0 && l < L - 1 && l != first_test) {
+          if (tid < QG && sh.qk[tid] > 0)
+            sh.qterm.S[tid] = a.eps * a.qtail[(int64_t)sh.qid[tid] * (L + 1) + l + 1];
+        } else if (l > 0 && tid < QG && sh.qk[tid] > 0) {
           const int q = sh.qid[tid];
           const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, sh.qk[tid]);
           const float tau = key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f);
           set_query_terms(tid, fminf(tau, __ldcg(a.tau_seed + q)),
-                          a.eps * a.qtail[(int64_t)q * (L + 1) + l + 1], sh.qterm[parity]);
+                          a.eps * a.qtail[(int64_t)q * (L + 1) + l + 1], sh.qterm);
         }
         if ((bad = epi_or(!ok || failed(fail)))) break;
-        const QTerms& qt = sh.qterm[parity];
-        parity ^= 1;
+        const QTerms& qt = sh.qterm;
 #pragma unroll 1
         for (uint32_t m = test; m; m &= m - 1) {
           const int c = __ffs(m) - 1;
@@ -1156,7 +1160,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
           if ((bad = epi_or(failed(fail)))) break;
         }
         if (bad) break;
-        QTerms& qt = sh.qterm[0];
+        QTerms& qt = sh.qterm;
         if (tightened) {
           if (tid < G && sh.qk[tid] > 0) set_query_terms(tid, sh.qtau[tid], 0.f, qt);
           if ((bad = epi_or(failed(fail)))) break;
