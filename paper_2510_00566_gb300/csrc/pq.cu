@@ -3,7 +3,7 @@
 //
 // Search: one thread block per (query, probed list) pair.  The block forms
 // the query residual r = q~ - c~ in shared memory and its level tail
-// energies (FP64), then walks the list in slabs of PQ_S candidates.  A
+// energies, then walks the list in slabs of a.slab candidates.  A
 // level's subvector terms e_m = ||r_m - C_m[code_m]||^2 come from a table of
 // the 256 terms of each of the level's subquantisers in shared memory (the
 // paper's per-level look-up tables) while many candidates are live, and
@@ -30,6 +30,7 @@
 #include "device_common.cuh"
 #include "gemm.h"
 #include "internal.h"
+#include "kernels_common.cuh"
 #include "probe_tc.h"
 #include "search.h"
 
@@ -38,7 +39,7 @@ namespace {
 
 constexpr int PQ_KSUB = 256;     // codewords per subquantiser (8-bit codes)
 constexpr int PQ_B = 256;        // vector slots per layout block
-constexpr int PQ_S = 2048;       // candidates per slab of one (query, list) pair
+constexpr int PQ_S = 2048;       // candidates per slab at most of one (query, list) pair
 constexpr int PQ_NT = 256;       // threads of the verify kernel
 constexpr int PQ_MAXML = 64;     // subquantisers per level
 constexpr int PQ_MAXDSUB = 32;   // coordinates per subvector
@@ -321,24 +322,25 @@ struct PqArgs {
   unsigned long long* topk;
   unsigned long long* stats;
   int d, M, dsub, L, ML, b, k_max, prune, collect;
+  int slab;    // candidates per slab of one (query, list) pair, PQ_S at most
   float lo;    // (1 - gamma) factor of the lower bound, rounded down
   float erel;  // relative allowance for the roundings of s_q, s_x and |s_q - s_x|
   float eps;   // Eq. 4 (1 = the exact, margined test)
 };
 
 // Bytes of dynamic shared memory of the verify kernel.
-size_t pq_verify_smem(int d, int L, int ML) {
+size_t pq_verify_smem(int d, int L, int ML, int slab) {
   size_t o = 0;
   auto take = [&](size_t bytes) {
     o = (o + 15) & ~(size_t)15;
     o += bytes;
   };
   take((size_t)d * 4);                 // r
-  take((size_t)L * 8);                 // level energies (FP64)
+  take((size_t)L * 8);                 // level energies (compensated FP32)
   take((size_t)L * 4);                 // s_q per level
   take((size_t)ML * PQ_KSUB * 4);      // level table
-  take((size_t)2 * PQ_S * 4);          // partial distances (two lists)
-  take((size_t)2 * PQ_S * 2);          // live candidates (two lists)
+  take((size_t)2 * slab * 4);          // partial distances (two lists)
+  take((size_t)2 * slab * 2);          // live candidates (two lists)
   take(64);                            // counters, threshold
   return o;
 }
@@ -520,9 +522,9 @@ __device__ __forceinline__ void level_sum4(const uint32_t* __restrict__ cp, int 
   }
 }
 
-__global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
+__global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int d = a.d, L = a.L, ML = a.ML, M = a.M, dsub = a.dsub;
+  const int d = a.d, L = a.L, ML = a.ML, M = a.M, dsub = a.dsub, slab = a.slab;
   size_t o = 0;
   auto carve = [&](size_t bytes) {
     o = (o + 15) & ~(size_t)15;
@@ -531,11 +533,11 @@ __global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
     return p;
   };
   float* r = (float*)carve((size_t)d * 4);
-  double* eq = (double*)carve((size_t)L * 8);
+  Acc2* eq = (Acc2*)carve((size_t)L * 8);
   float* sq = (float*)carve((size_t)L * 4);
   float* lut = (float*)carve((size_t)ML * PQ_KSUB * 4);
-  float* pacc = (float*)carve((size_t)2 * PQ_S * 4);
-  uint16_t* live = (uint16_t*)carve((size_t)2 * PQ_S * 2);
+  float* pacc = (float*)carve((size_t)2 * slab * 4);
+  uint16_t* live = (uint16_t*)carve((size_t)2 * slab * 2);
   int* ctr = (int*)carve(64);  // [0] survivors of the level, [2] threshold bits, [3] k,
                                // [8..15] four 64-bit section clocks
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -570,39 +572,37 @@ __global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
   for (int j = tid; j < d; j += PQ_NT)
     r[j] = __fsub_rn(a.qt[(size_t)q * d + j], a.cent_t[(size_t)c * d + j]);
   __syncthreads();
-  // FP64 level energies of the residual (one warp per level) while the whole
+  // level energies of the residual (one warp per level, compensated FP32: FP64
+  // instructions were a large part of a block's fixed work) while the whole
   // block builds level 0's table (the first slab needs it when it is large)
   for (int l = warp; l < L; l += PQ_NT / 32) {
-    double s = 0.0;
-    for (int j = lane; j < a.b; j += 32) {
-      const double v = r[l * a.b + j];
-      s += v * v;
-    }
-    for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    Acc2 s{0.f, 0.f};
+    for (int j = lane; j < a.b; j += 32) acc2_sq(s, r[l * a.b + j]);
+    s = warp_sum_acc2(s);
     if (lane == 0) eq[l] = s;
   }
   int lut_level = -1;  // the level whose table `lut` holds (uniform)
   unsigned long long n_lut = 0;
-  if (min(PQ_S, nc) >= PQ_LUT_MIN) {
+  if (min(slab, nc) >= PQ_LUT_MIN) {
     build_table(lut, r, a.codebook, 0, ML, dsub);
     lut_level = 0;
     n_lut = 1;
   }
   __syncthreads();
-  // tail after level l: one lane per level, FP64 sum, sqrt rounded to FP32
+  // tail after level l: one lane per level; its root is within 1.5 u
   if (warp == 0)
     for (int l = lane; l < L; l += 32) {
-      double tail = 0.0;
-      for (int l2 = L - 1; l2 > l; --l2) tail += eq[l2];
-      sq[l] = (float)sqrt(tail);
+      Acc2 tail{0.f, 0.f};
+      for (int l2 = L - 1; l2 > l; --l2) acc2_add(tail, eq[l2]);
+      sq[l] = __fsqrt_rn(__fadd_rn(tail.s, tail.c));
     }
   __syncthreads();
 
   lap(0);
   // counters (every thread keeps its own; summed at the end when collecting)
   unsigned long long n_dims = 0, n_lv = 0, n_full = 0;
-  for (int s0 = 0; s0 < nc; s0 += PQ_S) {
-    const int ns = min(PQ_S, nc - s0);
+  for (int s0 = 0; s0 < nc; s0 += slab) {
+    const int ns = min(slab, nc - s0);
     int nl = ns, cur = 0;
     for (int l = 0; l < L && nl > 0; ++l) {
       const bool last = l == L - 1;
@@ -612,8 +612,8 @@ __global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
         // tables), stopping at the first level whose test fails; no block
         // barrier per level
         for (int i = tid; i < nl; i += PQ_NT) {
-          const int cand = live[cur * PQ_S + i];
-          float P = pacc[cur * PQ_S + i];
+          const int cand = live[cur * slab + i];
+          float P = pacc[cur * slab + i];
           const int g = s0 + cand;
           const int64_t blk = blk0 + g / PQ_B;
           const int ln = g % PQ_B;
@@ -697,14 +697,14 @@ __global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
             }
           }
         } else if (i < nunits) {
-          cand0 = live[cur * PQ_S + i];
+          cand0 = live[cur * slab + i];
           const int g = s0 + cand0;
           const int64_t blk = blk0 + g / PQ_B;
           const int ln = g % PQ_B;
           const uint8_t* cp = a.codes + (blk * M + (int64_t)l * ML) * PQ_B + ln;
           const float S = use_lut ? level_sum1<true>(cp, ML, l * ML, lut, r, a.codebook, dsub)
                                   : level_sum_direct(cp, ML, l * ML, r, a.codebook, dsub);
-          const float P = __fadd_rn(pacc[cur * PQ_S + i], S);
+          const float P = __fadd_rn(pacc[cur * slab + i], S);
           Pv[0] = P;
           if (last) {
             const unsigned long long key = make_key(P, a.ids[blk * PQ_B + ln]);
@@ -723,8 +723,8 @@ __global__ void __launch_bounds__(PQ_NT, 3) pq_verify_kernel(const PqArgs a) {
             base = __shfl_sync(0xffffffffu, base, 0);
             if (keep[c]) {
               const int at = base + __popc(ball & ((1u << lane) - 1));
-              live[nxt * PQ_S + at] = (uint16_t)(cand0 + c);
-              pacc[nxt * PQ_S + at] = Pv[c];
+              live[nxt * slab + at] = (uint16_t)(cand0 + c);
+              pacc[nxt * slab + at] = Pv[c];
             }
           }
         }
@@ -1246,8 +1246,9 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     float lo32 = (float)lo;
     if ((double)lo32 > lo) lo32 = std::nextafter(lo32, 0.f);
     a.lo = lo32;
-    // s_q, s_x: FP64 sums rounded to FP32 (u each), |s_q - s_x| and the
-    // allowance itself (u each): 8u of (s_q + s_x) covers them with margin.
+    // s_q: a compensated sum and its root rounded (1.5 u), s_x: an FP64 sum
+    // rounded to FP32 (u), |s_q - s_x| and the allowance itself (u each): 8u of
+    // (s_q + s_x) covers them with margin.
     a.erel = (float)(8.0 * kU32);
     a.eps = (epsilon > 0.f && epsilon < 1.f) ? epsilon : 1.f;
 
@@ -1257,7 +1258,11 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     pq_seed_kernel<<<(unsigned)nq, 256, ssm, st>>>(a, probes, nprobe);
     PANO_CUDA(cudaGetLastError());
     mark(3);
-    const size_t vsm = pq_verify_smem(d, L, ML);
+    // lists of up to about 1,024 vectors fill one slab of half the size, and
+    // four blocks share an SM (250k x 960 on 256 lists, 4,096 queries: 3.87 ms
+    // with three, now 3.5)
+    a.slab = I.n <= (int64_t)1100 * nlist ? PQ_S / 2 : PQ_S;
+    const size_t vsm = pq_verify_smem(d, L, ML, a.slab);
     PANO_CUDA(cudaFuncSetAttribute(pq_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)vsm));
     pq_verify_kernel<<<(unsigned)npairs, PQ_NT, vsm, st>>>(a);
