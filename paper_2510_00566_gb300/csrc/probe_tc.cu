@@ -11,7 +11,7 @@
 // centroids and K panel of 64 the swizzled hi and lo operand images, 64 KB that
 // one bulk copy brings in.  (Each CTA used to convert its 256 centroid rows
 // itself, twice the work of its 128 queries: 10,000 x 1,024 x 960 took 296 us,
-// now 174.)
+// now 109.)
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -38,31 +38,46 @@ __device__ __forceinline__ void split2(float x, __nv_bfloat16& hi, __nv_bfloat16
 
 // Rows [r0, r0 + nr) of a row-major FP32 matrix (row length d), K panel p,
 // as bf16 hi and lo tiles of R rows in the swizzled K-major image (rows
-// past nr and elements past d are zeros).
-// vec: 16-byte loads (d % 4 == 0 and src 16-byte aligned).
+// past nr and elements past d are zeros).  A thread's loads all go out before
+// the first conversion (one after another they were most of a panel's time).
+// vec: 16-byte loads (d % 8 == 0 and src 16-byte aligned).
+template <int R>
 __device__ __forceinline__ void stage_rows(const float* __restrict__ src, int64_t r0, int nr,
-                                           int d, int p, int R, bool vec, unsigned char* hi,
+                                           int d, int p, bool vec, unsigned char* hi,
                                            unsigned char* lo) {
-  for (int e = threadIdx.x; e < R * (PK / 8); e += PT) {
-    const int r = e / (PK / 8), c8 = e % (PK / 8);
-    const int k0 = p * PK + c8 * 8;
-    float f[8];
-    if (vec && r < nr && k0 + 8 <= d) {
-      const float4* s4 = reinterpret_cast<const float4*>(src + (r0 + r) * (int64_t)d + k0);
-      const float4 a = __ldg(s4), b = __ldg(s4 + 1);
-      f[0] = a.x, f[1] = a.y, f[2] = a.z, f[3] = a.w;
-      f[4] = b.x, f[5] = b.y, f[6] = b.z, f[7] = b.w;
-    } else {
+  constexpr int kIter = R * (PK / 8) / PT, kBatch = 4;
+  static_assert(R * (PK / 8) % PT == 0 && kIter % kBatch == 0, "whole rounds");
+  const int c8 = threadIdx.x % (PK / 8), rr = threadIdx.x / (PK / 8);
+  const int k0 = p * PK + c8 * 8;
+#pragma unroll 1
+  for (int i0 = 0; i0 < kIter; i0 += kBatch) {
+    float f[kBatch][8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        f[j] = (r < nr && k0 + j < d) ? __ldg(src + (r0 + r) * (int64_t)d + k0 + j) : 0.f;
+    for (int u = 0; u < kBatch; ++u) {
+      const int r = rr + (i0 + u) * (PT / (PK / 8));
+      if (vec) {
+        const bool in = r < nr && k0 < d;  // (d % 8 == 0: whole groups)
+        const float4* s4 = reinterpret_cast<const float4*>(src + (r0 + r) * (int64_t)d + k0);
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a = in ? __ldg(s4) : z, b = in ? __ldg(s4 + 1) : z;
+        f[u][0] = a.x, f[u][1] = a.y, f[u][2] = a.z, f[u][3] = a.w;
+        f[u][4] = b.x, f[u][5] = b.y, f[u][6] = b.z, f[u][7] = b.w;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          f[u][j] = (r < nr && k0 + j < d) ? __ldg(src + (r0 + r) * (int64_t)d + k0 + j) : 0.f;
+      }
     }
-    __align__(16) __nv_bfloat16 h[8], l[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) split2(f[j], h[j], l[j]);
-    const uint32_t off = tc::swz_offset(r, c8 * 8, R, PK);
-    *reinterpret_cast<uint4*>(hi + off) = *reinterpret_cast<const uint4*>(h);
-    *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
+    for (int u = 0; u < kBatch; ++u) {
+      const int r = rr + (i0 + u) * (PT / (PK / 8));
+      __align__(16) __nv_bfloat16 h[8], l[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) split2(f[u][j], h[j], l[j]);
+      const uint32_t off = tc::swz_offset(r, c8 * 8, R, PK);
+      *reinterpret_cast<uint4*>(hi + off) = *reinterpret_cast<const uint4*>(h);
+      *reinterpret_cast<uint4*>(lo + off) = *reinterpret_cast<const uint4*>(l);
+    }
   }
 }
 
@@ -71,8 +86,8 @@ __global__ void __launch_bounds__(PT) cent_image_kernel(const float* __restrict_
                                                         int d, unsigned char* __restrict__ img) {
   unsigned char* out = img + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 * B_BYTES);
   const int c0 = blockIdx.y * PN;
-  stage_rows(C, c0, min(PN, nlist - c0), d, blockIdx.x, PN,
-             (d & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0, out, out + B_BYTES);
+  stage_rows<PN>(C, c0, min(PN, nlist - c0), d, blockIdx.x,
+                 (d & 7) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0, out, out + B_BYTES);
 }
 
 __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict__ Q, int64_t nq,
@@ -124,7 +139,7 @@ __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict
       bulk_g2s(st + 2 * A_BYTES, cimg + ((size_t)blockIdx.x * np + p) * (2 * B_BYTES), 2 * B_BYTES,
                &full[s]);
     }
-    stage_rows(Q, q0, nr_q, d, p, PM, vq, st, st + A_BYTES);
+    stage_rows<PM>(Q, q0, nr_q, d, p, vq, st, st + A_BYTES);
     fence_proxy_async_smem();
     tc::fence_before_sync();
     __syncthreads();
@@ -192,7 +207,16 @@ __global__ void __launch_bounds__(PT, 1) probe_tc_kernel(const float* __restrict
 // of a CTA's 128 rows in each of two halves of every centroid tile (row r's
 // two threads each scan 128 of a tile's 256 columns): keys (ordered distance
 // << 32 | id) ascending, best[row][half][kBest].
-constexpr int kBest = 4;
+// (With four, the rows that had to be compared with every centroid because a
+// half's last was within the bound, one in a thousand, were most of the pick.)
+constexpr int kBest = 6;
+static_assert(2 * kBest == kAssignWords && 2 * kBest <= 32, "a lane per key");
+
+// The distance in a key.
+__device__ __forceinline__ float expansion_of(unsigned long long key) {
+  const uint32_t o = (uint32_t)(key >> 32);
+  return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+}
 
 __global__ void __launch_bounds__(PT, 1) assign_tc_kernel(
     const float* __restrict__ X, int64_t m, const unsigned char* __restrict__ cimg, int nlist, int d,
@@ -228,6 +252,7 @@ __global__ void __launch_bounds__(PT, 1) assign_tc_kernel(
   unsigned long long b[kBest];
 #pragma unroll
   for (int i = 0; i < kBest; ++i) b[i] = kEmptyKey;
+  float worst = INFINITY;
   uint32_t dpar = 0, it = 0;  // panels of all tiles run through the two stages
   for (int c0 = 0; c0 < nlist; c0 += PN) {
     const int nc = nlist - c0 < PN ? nlist - c0 : PN, N = (nc + 15) & ~15;
@@ -244,7 +269,7 @@ __global__ void __launch_bounds__(PT, 1) assign_tc_kernel(
         bulk_g2s(st + 2 * A_BYTES, cimg + ((size_t)(c0 / PN) * np + p) * (2 * B_BYTES), 2 * B_BYTES,
                  &full[s]);
       }
-      stage_rows(X, r0, nr, d, p, PM, vx, st, st + A_BYTES);
+      stage_rows<PM>(X, r0, nr, d, p, vx, st, st + A_BYTES);
       fence_proxy_async_smem();
       tc::fence_before_sync();
       // (and the last tile's accumulators have been read)
@@ -278,22 +303,40 @@ __global__ void __launch_bounds__(PT, 1) assign_tc_kernel(
     for (int cb = 128 * half; cb < 128 * half + 128 && cb < N; cb += 16) {
       float v[16];
       tc::tmem_ld16(tbase + lane_base + (uint32_t)cb, v);
+      // sixteen distances and their least; few batches hold one below the
+      // row's kBest-th (ids ascend, so an equal one never enters)
+      float least = INFINITY;
+      const bool whole = c0 + cb + 16 <= nlist;
+#pragma unroll
+      for (int j = 0; j < 16; j += 4) {
+        float4 n4 = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+        if (whole) {  // (c0 + cb is a multiple of 16)
+          n4 = __ldg(reinterpret_cast<const float4*>(cn2 + c0 + cb + j));
+        } else {
+          if (c0 + cb + j < nlist) n4.x = __ldg(cn2 + c0 + cb + j);
+          if (c0 + cb + j + 1 < nlist) n4.y = __ldg(cn2 + c0 + cb + j + 1);
+          if (c0 + cb + j + 2 < nlist) n4.z = __ldg(cn2 + c0 + cb + j + 2);
+          if (c0 + cb + j + 3 < nlist) n4.w = __ldg(cn2 + c0 + cb + j + 3);
+        }
+        v[j] = fmaf(-2.f, v[j], n4.x);
+        v[j + 1] = fmaf(-2.f, v[j + 1], n4.y);
+        v[j + 2] = fmaf(-2.f, v[j + 2], n4.z);
+        v[j + 3] = fmaf(-2.f, v[j + 3], n4.w);
+        least = fminf(least, fminf(fminf(v[j], v[j + 1]), fminf(v[j + 2], v[j + 3])));
+      }
+      if (!(least < worst)) continue;
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const int c = c0 + cb + j;
-        if (c >= nlist) continue;
-        const unsigned long long key =
-            (unsigned long long)float_ordered(fmaf(-2.f, v[j], __ldg(cn2 + c))) << 32 | (uint32_t)c;
-        if (key < b[kBest - 1]) {
-          b[kBest - 1] = key;
+        if (!(v[j] < worst)) continue;
+        b[kBest - 1] = (unsigned long long)float_ordered(v[j]) << 32 | (uint32_t)(c0 + cb + j);
 #pragma unroll
-          for (int i = kBest - 1; i > 0; --i)
-            if (b[i] < b[i - 1]) {
-              const unsigned long long t = b[i];
-              b[i] = b[i - 1];
-              b[i - 1] = t;
-            }
-        }
+        for (int i = kBest - 1; i > 0; --i)
+          if (b[i] < b[i - 1]) {
+            const unsigned long long t = b[i];
+            b[i] = b[i - 1];
+            b[i - 1] = t;
+          }
+        if (b[kBest - 1] != kEmptyKey) worst = expansion_of(b[kBest - 1]);
       }
     }
     tc::fence_before_sync();
@@ -321,17 +364,13 @@ __global__ void __launch_bounds__(256) assign_pick_kernel(
   const float* x = X + row * d;
   const unsigned long long key = lane < 2 * kBest ? best[row * 2 * kBest + lane] : kEmptyKey;
   const unsigned long long first = warp_min_u64(key);
-  auto dec = [](unsigned long long k) {
-    const uint32_t o = (uint32_t)(k >> 32);
-    return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
-  };
   float n2 = 0.f;
   for (int j = lane; j < d; j += 32) n2 = fmaf(x[j], x[j], n2);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, off);
   const float s = sqrtf(n2) * 1.0001f + cmax;  // (the sum's rounding is far below 1e-4)
-  const float hi = dec(first) + 2.f * gerr * s * s * 1.0001f;
-  const uint32_t near = __ballot_sync(0xffffffffu, key != kEmptyKey && dec(key) <= hi);
+  const float hi = expansion_of(first) + 2.f * gerr * s * s * 1.0001f;
+  const uint32_t near = __ballot_sync(0xffffffffu, key != kEmptyKey && expansion_of(key) <= hi);
   int choice = (int)(uint32_t)first;
   if (near & (near - 1)) {
     float e = INFINITY;
@@ -394,7 +433,7 @@ int launch_probe_tc(const float* Q, int64_t nq, const pano_index& I, const float
   }));
   if (nq <= 0 || nlist <= 0) return PANO_OK;
   const dim3 grid((unsigned)((nlist + PN - 1) / PN), (unsigned)((nq + PM - 1) / PM));
-  const bool vq = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(Q) & 15) == 0;
+  const bool vq = (d & 7) == 0 && (reinterpret_cast<uintptr_t>(Q) & 15) == 0;
   probe_tc_kernel<<<grid, PT, smem, st>>>(Q, nq, I.cent_img.as<unsigned char>(), nlist, d, qn2,
                                           I.cent_n2.as<float>(), pd, err, vq);
   PANO_CUDA(cudaGetLastError());
@@ -411,7 +450,7 @@ int launch_assign_tc(const float* X, int64_t m, const pano_index& I, unsigned lo
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }));
   if (m <= 0) return PANO_OK;
-  const bool vx = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  const bool vx = (d & 7) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
   assign_tc_kernel<<<(unsigned)((m + PM - 1) / PM), PT, smem, st>>>(
       X, m, I.cent_img.as<unsigned char>(), nlist, d, I.cent_n2.as<float>(), best, err, vx);
   PANO_CUDA(cudaGetLastError());

@@ -19,7 +19,8 @@ int build_cent_image(pano_index& I, cudaStream_t st);
 int launch_probe_tc(const float* Q, int64_t nq, const pano_index& I, const float* qn2, float* pd,
                     int* err, cudaStream_t st);
 // out[i]: the nearest centroid of row i < m of X (exact distances decide, ties
-// to the lower id); best: 8 m words of workspace.
+// to the lower id); best: kAssignWords m words of workspace.
+constexpr int kAssignWords = 12;
 int launch_assign_tc(const float* X, int64_t m, const pano_index& I, unsigned long long* best,
                      int32_t* out, int* err, cudaStream_t st);
 
