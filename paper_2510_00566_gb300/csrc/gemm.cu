@@ -266,6 +266,29 @@ __global__ void __launch_bounds__(NT, 2) gemm_nt64_kernel(int M, int N, int K,
   }
 }
 
+// A few rows (kStoreAny, M <= kRowsMax): one warp per (row, column), the lanes
+// along K, so that every SM has a part of B to read; the 128 x 64 tiles left all
+// but N / 64 of them idle (one query of 960: 298 us a search, 244 so with
+// the seeds below 152 queries).  A product
+// passes through ceil(K / 32) + 6 roundings at most, fewer than in the tiles.
+constexpr int kRowsMax = 8;
+
+__global__ void __launch_bounds__(NT) gemm_rows_kernel(int N, int K, const float* __restrict__ A,
+                                                       int lda, const float* __restrict__ mu,
+                                                       const float* __restrict__ B, int ldb,
+                                                       float* __restrict__ C, int64_t ldc) {
+  const int n = blockIdx.x * (NT / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
+  if (n >= N) return;
+  const float* a = A + (int64_t)blockIdx.y * lda;
+  const float* b = B + (int64_t)n * ldb;
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = lane; k < K; k += 32) s = fmaf(a[k] - (mu ? mu[k] : 0.f), b[k], s);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) C[(int64_t)blockIdx.y * ldc + n] = s;
+}
+
 __device__ __forceinline__ void top2_push(unsigned long long& k0, unsigned long long& k1,
                                           unsigned long long key) {
   if (key < k0) {
@@ -332,13 +355,18 @@ cudaError_t gemm_nt(int mode, int M, int N, int K, const float* A, int lda, cons
                     const float* B, int ldb, float* C, int64_t ldc, const float* an,
                     const float* bn, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  if (mode == kStoreAny && M <= kRowsMax) {
+    const dim3 g((N + NT / 32 - 1) / (NT / 32), M);
+    gemm_rows_kernel<<<g, NT, 0, st>>>(N, K, A, lda, mu, B, ldb, C, ldc);
+    return cudaGetLastError();
+  }
   dim3 grid((M + BM - 1) / BM, (N + BN2 - 1) / BN2);
   if (grid.y > 65535) return cudaErrorInvalidValue;
   // float4 loads need 16-byte aligned rows (and mu)
   const bool vec = ((K | lda | ldb) & 3) == 0 && ((uintptr_t)A & 15) == 0 &&
                    ((uintptr_t)B & 15) == 0 && ((uintptr_t)mu & 15) == 0;
   const size_t sm = sizeof(Tile2);  // 25.3 KB
-  if (mode == kStore) {
+  if (mode != kDist) {
     if (vec)
       gemm_nt64_kernel<kStore, true><<<grid, NT, sm, st>>>(M, N, K, A, lda, mu, B, ldb, C, ldc, an, bn);
     else

@@ -7,9 +7,11 @@
 
 namespace pano {
 
-enum { kStore = 0, kDist = 1 };
+// kStoreAny: kStore where the sums' order may depend on M (the query transform,
+// whose rounding only moves bounds; IVFPQ's distances keep one order).
+enum { kStore = 0, kDist = 1, kStoreAny = 2 };
 
-// C[m][n] = sum_k (A[m][k] - mu[k]) * B[n][k]      (mode kStore; mu may be 0)
+// C[m][n] = sum_k (A[m][k] - mu[k]) * B[n][k]      (modes kStore, kStoreAny; mu may be 0)
 // C[m][n] = an[m] + bn[n] - 2 * sum_k A[m][k] B[n][k]   (mode kDist)
 cudaError_t gemm_nt(int mode, int M, int N, int K, const float* A, int lda, const float* mu,
                     const float* B, int ldb, float* C, int64_t ldc, const float* an,
