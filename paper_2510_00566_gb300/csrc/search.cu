@@ -502,7 +502,10 @@ __device__ __forceinline__ int seed_count(int n, int k) {
 }
 constexpr int kSeedWarps = 8;
 
-__global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
+// W warps: 8, or 16 for a batch too small to fill the SMs (its rounds of rows are
+// waited for one after another).
+template <int W>
+__global__ void __launch_bounds__(W * 32) seed_tau_kernel(
     const float* __restrict__ q, int d, const int32_t* __restrict__ probes, int stride,
     const int64_t* __restrict__ chunk_off, const int32_t* __restrict__ list_size, int chunk,
     const float* __restrict__ rows, const int32_t* __restrict__ kq,
@@ -521,12 +524,12 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
     return;
   }
   float* qs = reinterpret_cast<float*>(qs4);
-  for (int j = threadIdx.x; j < d; j += kSeedWarps * 32) qs[j] = q[row * d + j];
+  for (int j = threadIdx.x; j < d; j += W * 32) qs[j] = q[row * d + j];
   __syncthreads();
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
   const int64_t base = chunk_off[c] * chunk;  // a list's members are its first slots
   const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(rows) & 15) == 0;
-  for (int i = warp; i < ns; i += kSeedWarps) {
+  for (int i = warp; i < ns; i += W) {
     const float* x = rows + (base + i) * d;
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     if (vec) {
@@ -590,7 +593,7 @@ __global__ void __launch_bounds__(kSeedWarps * 32) seed_tau_kernel(
   __syncthreads();
   if (!topk) return;
   const float t = s_t;
-  for (int i = warp; i < ns; i += kSeedWarps) {
+  for (int i = warp; i < ns; i += W) {
     if (!(dist[i] <= t)) continue;
     const float e = exact_sqdist_warp_wide(q + row * d, rows + (base + i) * d, d);
     topk_insert_warp(topk + row * k_max, k, make_key(e, ids[base + i]));
@@ -1840,7 +1843,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     PANO_CUDA(cudaGetLastError());
     // a1
     mark(0);
-    PANO_CUDA(gemm_nt(kStore, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(), d,
+    PANO_CUDA(gemm_nt(kStoreAny, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(), d,
                       qt, d, nullptr, nullptr, st));
     const int split = I.precision == PANO_BF16  ? kSplitBf16
                       : I.precision == PANO_FP8 ? kSplitE4m3
@@ -1928,7 +1931,8 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
           I.list_size_d.as<int32_t>(), I.chunk, I.rows.as<float>(), kq, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     } else {
-      seed_tau_kernel<<<(unsigned)nq, kSeedWarps * 32, (size_t)d * 4, st>>>(
+      auto seeds = nq < 152 ? seed_tau_kernel<16> : seed_tau_kernel<kSeedWarps>;
+      seeds<<<(unsigned)nq, (nq < 152 ? 16 : kSeedWarps) * 32, (size_t)d * 4, st>>>(
           queries, d, probes, stride, I.chunk_off_d.as<int64_t>(), I.list_size_d.as<int32_t>(),
           I.chunk, I.rows.as<float>(), kq, one_pass ? nullptr : bucket, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
@@ -2195,7 +2199,7 @@ int transform_queries(const pano_index& I, const float* queries, int64_t nq, flo
                       float4* qinfo, float* qtail, float* qn2, cudaStream_t st) {
   const int d = I.d, L = I.L;
   if (nq == 0) return PANO_OK;
-  PANO_CUDA(gemm_nt(kStore, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(), d,
+  PANO_CUDA(gemm_nt(kStoreAny, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(), d,
                     qt, d, nullptr, nullptr, st));
   float c_trans_up = (float)I.c_trans;
   if ((double)c_trans_up < I.c_trans) c_trans_up = std::nextafter(c_trans_up, INFINITY);
