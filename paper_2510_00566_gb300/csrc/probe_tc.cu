@@ -371,8 +371,10 @@ __global__ void __launch_bounds__(256) assign_pick_kernel(
   const float s = sqrtf(n2) * 1.0001f + cmax;  // (the sum's rounding is far below 1e-4)
   const float hi = expansion_of(first) + 2.f * gerr * s * s * 1.0001f;
   const uint32_t near = __ballot_sync(0xffffffffu, key != kEmptyKey && expansion_of(key) <= hi);
-  int choice = (int)(uint32_t)first;
-  if (near & (near - 1)) {
+  // A norm beyond FP32 (or NaN) makes the expansion the same for every centroid:
+  // the lowest id, as from the FP32 products; so too where no key was kept.
+  int choice = first == kEmptyKey || !(n2 < INFINITY) ? 0 : (int)(uint32_t)first;
+  if (n2 < INFINITY && (near & (near - 1))) {
     float e = INFINITY;
     int c = nlist;
     auto look = [&](int ci) {
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(256) assign_pick_kernel(
       for (uint32_t k = near; k; k &= k - 1)
         look((int)(uint32_t)__shfl_sync(0xffffffffu, key, __ffs(k) - 1));
     }
-    choice = c;
+    if (c < nlist) choice = c;  // (no distance compares where a centroid is not finite)
   }
   if (lane == 0) out[row] = choice;
 }
