@@ -190,14 +190,17 @@ __global__ void __launch_bounds__(256) pack_fp32_kernel(
       Acc2 e{0.f, 0.f};
       if (valid)
         for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) acc2_sq(e, x[j]);
-      rb.level(l, e);
+      rb.level(l, warp_acc2_f64(e, level_off[l], level_off[l + 1],
+                                [&](int j) { return (double)x[j] * x[j]; }));
     }
     Acc2 dev{0.f, 0.f};  // ||x - mu~||
-    if (valid) {
-      const float* r = rows + (lc * CH + i) * (int64_t)d;  // rows of this block
+    const float* r = rows + (lc * CH + i) * (int64_t)d;  // rows of this block
+    if (valid)
       for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
-    }
-    const double de = acc2_f64(warp_sum_acc2(dev));
+    const double de = warp_acc2_f64(dev, 0, d, [&](int j) {
+      const double v = (double)r[j] - (double)mu[j];
+      return v * v;
+    });
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int l = lane + 32 * u;

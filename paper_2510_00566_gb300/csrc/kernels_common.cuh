@@ -339,6 +339,20 @@ __device__ __forceinline__ void acc2_sqdiff(Acc2& a, float x, float y) {
 
 __device__ __forceinline__ double acc2_f64(Acc2 a) { return (double)a.s + (double)a.c; }
 
+// The warp's total of a sum as FP64.  A sum that left FP32's range (elements
+// above 1.8e19) is formed again in FP64, from term(j) over j = lo .. hi - 1.
+template <class F>
+__device__ __forceinline__ double warp_acc2_f64(Acc2 a, int lo, int hi, F term) {
+  const double s = acc2_f64(warp_sum_acc2(a));
+  if (fabs(s) < INFINITY) return s;  // (the same in every lane)
+  double t = 0.0;
+#pragma unroll 1
+  for (int j = lo + (int)(threadIdx.x & 31); j < hi; j += 32) t += term(j);
+#pragma unroll 1
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+  return t;
+}
+
 // What a packed row's bounds are made of, by one warp: the level energies of
 // the stored vector summed from the last level backwards give the rounded-up
 // tail norms; qerr (the squared storage error) and dev (|x - mu~|^2) give e_x.
@@ -350,8 +364,8 @@ __device__ __forceinline__ double acc2_f64(Acc2 a) { return (double)a.s + (doubl
 struct RowBounds {
   double tail[2] = {0.0, 0.0};  // energies from level lane (and lane + 32) on
   double energy = 0.0;          // of the whole row
-  __device__ __forceinline__ void level(int l, Acc2 e) {
-    energy += acc2_f64(warp_sum_acc2(e));
+  __device__ __forceinline__ void level(int l, double e) {
+    energy += e;
     if (l == (int)(threadIdx.x & 31)) tail[0] = energy;
     if (l == (int)(threadIdx.x & 31) + 32) tail[1] = energy;
   }

@@ -594,7 +594,14 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
     for (int l = lane; l < L; l += 32) {
       Acc2 tail{0.f, 0.f};
       for (int l2 = L - 1; l2 > l; --l2) acc2_add(tail, eq[l2]);
-      sq[l] = __fsqrt_rn(__fadd_rn(tail.s, tail.c));
+      const float e = __fadd_rn(tail.s, tail.c);
+      if (e < INFINITY) {
+        sq[l] = __fsqrt_rn(e);
+      } else {  // beyond FP32's range: the sum again in FP64
+        double t = 0.0;
+        for (int j = (l + 1) * a.b; j < d; ++j) t += (double)r[j] * r[j];
+        sq[l] = (float)sqrt(t);
+      }
     }
   __syncthreads();
 
