@@ -96,18 +96,26 @@ __host__ __device__ __forceinline__ uint32_t idesc_e4m3(int M, int N) {
 }
 
 // ------------------------------------------------------------------ TMEM
+// The instructions below that end in .sync.aligned need all 32 lanes of a
+// converged warp.  A caller's lanes may have parted before (a loop that some
+// leave early, a wait that each polls for itself; a vote does not promise that
+// they rejoin), so each helper begins with a __syncwarp().
+
 // Allocate `ncols` (power of two >= 32) columns; the address is written to
 // *dst_smem.  Executed by one full warp.
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                    smem_u32(dst_smem)),
                "r"(ncols)
                : "memory");
 }
 __device__ __forceinline__ void tmem_relinquish() {
+  __syncwarp();
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
                : "memory");
 }
@@ -147,6 +155,7 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 // 32 consecutive f32 columns of this thread's TMEM lane (warp w reads lanes
 // 32*(w%4) .. +31; `taddr` carries the lane base in bits [16,32)).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+  __syncwarp();
   uint32_t r[32];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
@@ -165,6 +174,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 
 // 16 consecutive f32 columns (same lane rule).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+  __syncwarp();
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
@@ -180,6 +190,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 
 // 8 consecutive f32 columns (same lane rule).
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  __syncwarp();
   uint32_t r[8];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -193,6 +204,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
 
 // One f32 column (same lane rule).
 __device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+  __syncwarp();
   uint32_t r;
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
