@@ -220,10 +220,14 @@ __device__ __forceinline__ void topk_replace_warp(unsigned long long* slots, int
 #pragma unroll
       for (int r = 0; r < 4; ++r)
         v[r] = 32 * r + lane < k ? ld_volatile_u64(slots + 32 * r + lane) : 0ull;
-      // (an absent slot is 0: below every key, never the largest while k > 0)
+      // (an absent slot reads 0: never the largest of distinct keys while k > 1.
+      // It is also the key of id 0 at distance 0, so only slots that exist are
+      // compared below.)
       for (uint32_t m = __ballot_sync(0xffffffffu, key != kEmptyKey); m; m &= m - 1) {
         const unsigned long long x = __shfl_sync(0xffffffffu, key, __ffs(m) - 1);
-        const bool same = v[0] == x || v[1] == x || v[2] == x || v[3] == x;
+        bool same = false;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) same |= (32 * r + lane < k) & (v[r] == x);
         if (__any_sync(0xffffffffu, same) && lane == __ffs(m) - 1) dup = true;
       }
       if (dup) key = kEmptyKey;  // the pair is held already
