@@ -792,7 +792,6 @@ __global__ void __launch_bounds__(256) pq_seed_kernel(const PqArgs a,
   // code loads hit one 32-byte run per subquantiser
   for (int e = threadIdx.x; e < ns * L; e += blockDim.x) {
     const int cand = e % ns, l = e / ns;
-  if (c < 0) return;  // no list: the query's distances are NaN
     const int64_t blk = blk0 + cand / PQ_B;
     const int ln = cand % PQ_B;
     const uint8_t* cp = a.codes + (blk * a.M + (int64_t)l * ML) * PQ_B + ln;
@@ -833,8 +832,8 @@ __global__ void pq_pair_count_kernel(const int32_t* __restrict__ probes, int64_t
                                      const int32_t* __restrict__ kq, int* __restrict__ cnt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nq * nprobe || !pq_pair_live(i, nprobe, npq, kq)) return;
-  const int rank = (int)(i % nprobe), c = probes[i];
-  if (c >= 0) atomicAdd(cnt + (rank > 0) * nlist + c, 1);
+  const int rank = (int)(i % nprobe);
+  atomicAdd(cnt + (rank > 0) * nlist + probes[i], 1);
 }
 
 __global__ void __launch_bounds__(1024) pq_pair_scan_kernel(const int* __restrict__ cnt, int nb,
@@ -878,7 +877,6 @@ __global__ void pq_decode_kernel(const unsigned long long* __restrict__ topk, in
   if (i >= n) return;
   const unsigned long long key = topk[i];
   ids[i] = key == kEmptyKey ? -1 : (int64_t)key_id(key);
-  if (c < 0) return;
   dists[i] = key == kEmptyKey ? INFINITY : key_dist(key);
 }
 
