@@ -781,6 +781,7 @@ __global__ void __launch_bounds__(256) pq_seed_kernel(const PqArgs a,
   float* part = r + ((d + 3) & ~3);  // [PQ_SEED][L]
   const int q = blockIdx.x;
   const int c = probes[(size_t)q * nprobe];
+  if (c < 0) return;  // no list: the query's distances are NaN
   const int ns = min(PQ_SEED, a.list_size[c]);
   const int kq = a.kq[q];
   if (ns == 0 || kq == 0) return;
@@ -832,8 +833,8 @@ __global__ void pq_pair_count_kernel(const int32_t* __restrict__ probes, int64_t
                                      const int32_t* __restrict__ kq, int* __restrict__ cnt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nq * nprobe || !pq_pair_live(i, nprobe, npq, kq)) return;
-  const int rank = (int)(i % nprobe);
-  atomicAdd(cnt + (rank > 0) * nlist + probes[i], 1);
+  const int rank = (int)(i % nprobe), c = probes[i];
+  if (c >= 0) atomicAdd(cnt + (rank > 0) * nlist + c, 1);
 }
 
 __global__ void __launch_bounds__(1024) pq_pair_scan_kernel(const int* __restrict__ cnt, int nb,
@@ -866,6 +867,7 @@ __global__ void pq_pair_scatter_kernel(const int32_t* __restrict__ probes, int64
   if (i >= nq * nprobe || !pq_pair_live(i, nprobe, npq, kq)) return;
   const int rank = (int)(i % nprobe);
   const int c = probes[i];
+  if (c < 0) return;
   const int b = (rank > 0) * nlist + c;
   const int at = off[b] + atomicAdd(fill + b, 1);
   pairs[at] = make_int2((int)(i / nprobe), c);

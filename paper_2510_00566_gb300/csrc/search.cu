@@ -293,7 +293,9 @@ __global__ void __launch_bounds__(NT) probe_select_kernel(
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
   for (int b = b0 + warp; b < kBandCap; b += NT / 32) {
     float e = exact_sqdist_warp(q + row * d, cent + (int64_t)band_id[b] * d, d);
-    if (lane == 0) band_d[b] = e;
+    // (a distance beyond FP32 comes out as NaN, which has no rank: a place of
+    // the result would stay unwritten)
+    if (lane == 0) band_d[b] = e < INFINITY ? e : INFINITY;
   }
   __syncthreads();
   // ranks: below the band among themselves, the band among itself after them
@@ -318,7 +320,8 @@ __global__ void __launch_bounds__(NT) probe_select_kernel(
     }
     if (rank < m) out[rank] = ib;
   }
-  for (int r = ni + nb + threadIdx.x; r < m; r += NT) out[r] = -1;  // unreachable unless nlist < m
+  // no more lists: nlist < m, or NaN distances
+  for (int r = ni + nb + threadIdx.x; r < m; r += NT) out[r] = -1;
 }
 
 // ------------------------------------------------------- a3: work inversion
