@@ -161,20 +161,23 @@ __device__ __forceinline__ void topk_insert_warp(unsigned long long* slots, int 
     }
 }
 
-// A query with k above this keeps its slots unsorted: a new key replaces the
-// largest one (topk_replace_warp), and its threshold lives in tau_seed alone.
+// In a batch with unsorted slots (a rule on the host) a query with k above this
+// keeps its slots unsorted: a new key replaces the largest one
+// (topk_replace_warp), and its threshold lives in tau_seed alone.
 // With sorted slots a key costs up to k dependent global atomics (about 0.7 us
 // each); a replacement costs one round of loads and one of compare-exchanges
 // for up to 32 keys of a query.  At k = 10 the chains of a flush end sooner (a
 // warp takes its queries one after another); at k = 100 they were 84 % of the
 // verify kernel (1.5M x 384 BF16, Zipf lists, 16,384 queries, k in {1, 10,
-// 100}: 59 ms a search, 28 with a locked merge per flush, 20 so).  At k = 37
-// both take the same time.
+// 100}: 59 ms a search, 28 with a locked merge per flush, 20 so).  At k = 41
+// and 256 to 1,024 queries both take about the same time (200k x 128 BF16, nprobe
+// 8 of 128: 464 / 450 and 847 / 900 us a search).
 constexpr int kChainK = 40;
 
 // The k-th key of a query's sorted slots, kEmptyKey where they are unsorted.
+template <bool LARGE>
 __device__ __forceinline__ unsigned long long kth_key(const unsigned long long* slots, int k) {
-  return k <= kChainK ? ld_volatile_u64(slots + k - 1) : kEmptyKey;
+  return !LARGE || k <= kChainK ? ld_volatile_u64(slots + k - 1) : kEmptyKey;
 }
 
 // Smallest / largest 64-bit value of the warp.
@@ -291,8 +294,7 @@ __device__ __forceinline__ void topk_replace_warp(unsigned long long* slots, int
 // Enters the flush's pairs into their queries' top-k: entry i < n is pair
 // list[i], its distance dist[], id pid[] and query pq[].  Called by all
 // `nthreads` threads of the flush (tid 0 .. nthreads - 1, n <= nthreads),
-// between barriers.  LARGE = false: every k is at most kChainK (the batch's
-// k_max is).
+// between barriers.  LARGE = false: all slots of the batch are sorted.
 template <bool LARGE>
 __device__ __forceinline__ void topk_flush_insert(unsigned long long* topk, int k_max,
                                                   const int32_t* __restrict__ kq, float* tau_seed,

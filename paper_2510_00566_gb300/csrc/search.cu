@@ -829,7 +829,7 @@ __device__ __forceinline__ float sqrt_ratio_up(float tau, float inv_lb_up) {
 // Survivors are re-ranked in batches (those whose lower bound exceeds the
 // threshold by then are dropped); the delayed top-k insertions only leave
 // the threshold larger for a while, which is still a valid threshold.
-// LARGE: some k of the batch is above kChainK.
+// LARGE: the slots of queries with k > kChainK are unsorted.
 template <int QB, int CB, int NTH, int NST, bool LARGE>
 __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a) {
   constexpr int NCH = CB / CH;
@@ -995,7 +995,7 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
   auto read_tau = [&](int g, int G) {
     TauRead r{kEmptyKey, -1.f};  // k == 0: nothing can enter
     if (g < G && qk[g] > 0) {
-      r.key = kth_key(a.topk + (int64_t)qid[g] * a.k_max, qk[g]);
+      r.key = kth_key<LARGE>(a.topk + (int64_t)qid[g] * a.k_max, qk[g]);
       r.seed = __ldcg(a.tau_seed + qid[g]);
     }
     return r;
@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
     // k are closer; the pair's own upper bound is never below its lower one)
     for (int s = tid; s < np; s += NTH) {
       const int q = pq[s], kk = a.kq[q];
-      const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, kk);
+      const unsigned long long key = kth_key<LARGE>(a.topk + (int64_t)q * a.k_max, kk);
       const float tau = fminf(key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f),
                               __ldcg(a.tau_seed + q));
       const float lb = plb[s];
@@ -1508,7 +1508,8 @@ __global__ void __launch_bounds__(NTH, 2) verify_fp32_kernel(const VerifyArgs a)
   }
 }
 
-__global__ void decode_kernel(int64_t nq, int k_max, const int32_t* __restrict__ kq,
+// sorted_k: the largest k whose slots are sorted.
+__global__ void decode_kernel(int64_t nq, int k_max, int sorted_k, const int32_t* __restrict__ kq,
                               const unsigned long long* __restrict__ topk,
                               int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1517,7 +1518,7 @@ __global__ void decode_kernel(int64_t nq, int k_max, const int32_t* __restrict__
   int j = (int)(e % k_max);
   const int k = kq[qi];
   unsigned long long key = j < k ? topk[e] : kEmptyKey;
-  if (k > kChainK && j < k) {
+  if (k > sorted_k && j < k) {
     // unsorted slots: a key's place is the number of smaller ones (keys are
     // distinct), an empty slot's the keys plus the empty slots before it
     const unsigned long long* slots = topk + qi * k_max;
@@ -1651,13 +1652,31 @@ int pick_tile(const TileCfg* list, int n, int max_w, int L, TileCfg* out, int* b
   return fail(PANO_EINVAL, "verify tile does not fit in shared memory");
 }
 
+// Whether the slots of queries with k > kChainK are kept unsorted (see kChainK).
+// With few queries the chains win: a flush's keys run down the slots side by
+// side, a thread each, where replacements take them one after another, a warp
+// per query.  With many, the chains of all work items meet on the same slots.
+// Chains / replacements, us a search: 200k x 128 BF16, nprobe 8 of 128, k = 100:
+// one query 228 / 413, 32 394 / 493, 128 709 / 570, 1,024 1,985 / 1,581; 200k x
+// 768 FP8, nprobe 16 of 128 (more pairs reach re-ranking): 16 queries 729 / 830,
+// 64 1,391 / 1,144; 200k x 128 FP32: 32 queries 606 / 654, 128 1,126 / 920.
+// Above 128 results, where each replacement reads all slots again: BF16, k = 300
+// and nprobe 32 of 1,024, 128 queries 2,157 / 3,177, 512 5,043 / 5,215; FP32, 16
+// queries 2,187 / 1,772.
+bool unsorted_slots(int precision, int64_t nq, int k_max) {
+  if (k_max <= kChainK) return false;
+  if (precision == PANO_FP8) return nq >= 32;
+  if (k_max <= 128) return nq >= 128;
+  return nq >= (precision == PANO_FP32 ? 16 : 256);
+}
+
 // Launches the picked tile.  The grid is sized from the shared-memory plan,
 // not from the occupancy API, whose answer follows the SM's current
 // shared-memory carveout.
-int launch_verify(const VerifyArgs& a, const TileCfg& c, int bps, cudaStream_t st) {
+int launch_verify(const VerifyArgs& a, const TileCfg& c, int bps, bool large, cudaStream_t st) {
   const void* k = nullptr;
   size_t ss = 0;
-  PANO_CUDA(tile_attrs(c, a.k_max > kChainK, &k, &ss));
+  PANO_CUDA(tile_attrs(c, large, &k, &ss));
   int dev = 0, sms = 0;
   PANO_CUDA(cudaGetDevice(&dev));
   PANO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1942,6 +1961,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     }
     PANO_CUDA(cudaGetLastError());
     // a4-a10
+    const bool large = unsorted_slots(I.precision, nq, k_max);
     if (tcpath) {
       VerifyTCArgs ta;
       std::memset(&ta, 0, sizeof(ta));
@@ -2003,7 +2023,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       ta.counter = tot + 4;
       ta.items_cap = capA;
       ta.phase = 0;
-      int r = one_pass ? PANO_OK : launch_verify_tc(ta, st);  // one pass: phase A is empty
+      int r = one_pass ? PANO_OK : launch_verify_tc(ta, large, st);  // one pass: phase A is empty
       if (r) return r;
       mark(4);
       ta.items = itB;
@@ -2011,7 +2031,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
       ta.counter = tot + 5;
       ta.items_cap = capB;
       ta.phase = 1;
-      r = launch_verify_tc(ta, st);
+      r = launch_verify_tc(ta, large, st);
       if (r) return r;
     } else {
     VerifyArgs va;
@@ -2057,7 +2077,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     va.counter = tot + 4;
     va.items_cap = capA;
     va.phase = 0;
-    int r = one_pass ? PANO_OK : launch_verify(va, tileA, bpsA, st);  // one pass: phase A is empty
+    int r = one_pass ? PANO_OK : launch_verify(va, tileA, bpsA, large, st);  // one pass: phase A is empty
     if (r) return r;
     // phase B
     mark(4);
@@ -2066,13 +2086,13 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
     va.counter = tot + 5;
     va.items_cap = capB;
     va.phase = 1;
-    r = launch_verify(va, tileB, bpsB, st);
+    r = launch_verify(va, tileB, bpsB, large, st);
     if (r) return r;
     }
     mark(5);
     const int64_t no = nq * k_max;
-    decode_kernel<<<(unsigned)((no + 255) / 256), 256, 0, st>>>(nq, k_max, kq, topk, out_ids,
-                                                                out_dists);
+    decode_kernel<<<(unsigned)((no + 255) / 256), 256, 0, st>>>(nq, k_max, large ? kChainK : k_max,
+                                                                kq, topk, out_ids, out_dists);
     PANO_CUDA(cudaGetLastError());
     mark(6);
     // the device error word for a caller that does not synchronize (it maps

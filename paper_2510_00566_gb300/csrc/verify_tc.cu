@@ -433,7 +433,7 @@ __device__ __noinline__ int flush_pending(const VerifyTCArgs& a, Shared& sh, int
   if (tid < QG) sh.scount[tid] = 0;
   if (sync_failed()) return -1;
   auto tau_of = [&](int q, int kk) {
-    const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, kk);
+    const unsigned long long key = kth_key<LARGE>(a.topk + (int64_t)q * a.k_max, kk);
     return fminf(key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f),
                  __ldcg(a.tau_seed + q));
   };
@@ -558,9 +558,9 @@ __device__ __forceinline__ uint32_t stage_tag(uint32_t seq, int panel, int c) {
 // width), kind::f8f6f4 MMAs with the query split into three E4M3 terms at a
 // power-of-two scale of its own; the accumulator times the row's scale s_x and
 // the query's is the partial product.
-// LARGE: some k of the batch is above kChainK (the replacements of the flush
-// cost the level loop registers, so a batch without them runs without their
-// code).
+// LARGE: the slots of queries with k > kChainK are unsorted (the replacements
+// of the flush cost the level loop registers, so a batch without them runs
+// without their code).
 template <bool FP8, bool LARGE, int F>
 __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant__ VerifyTCArgs a) {
   using R = Ring<FP8, F>;
@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
           const unsigned b = __ballot_sync(0xffffffffu, kk > 0);
           if (lane == 0) sh.gm[warp] = b;
           if (kk > 0) {
-            const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, kk);
+            const unsigned long long key = kth_key<LARGE>(a.topk + (int64_t)q * a.k_max, kk);
             const float tau = key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f);
             set_query_terms(tid, fminf(tau, __ldcg(a.tau_seed + q)),
                             a.eps * a.qtail[(int64_t)q * (L + 1) + 1], sh.qterm);
@@ -1047,7 +1047,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
             sh.qterm.S[tid] = a.eps * a.qtail[(int64_t)sh.qid[tid] * (L + 1) + l + 1];
         } else if (l > 0 && tid < QG && sh.qk[tid] > 0) {
           const int q = sh.qid[tid];
-          const unsigned long long key = kth_key(a.topk + (int64_t)q * a.k_max, sh.qk[tid]);
+          const unsigned long long key = kth_key<LARGE>(a.topk + (int64_t)q * a.k_max, sh.qk[tid]);
           const float tau = key == kEmptyKey ? INFINITY : __fmul_ru(key_dist(key), 1.000001f);
           set_query_terms(tid, fminf(tau, __ldcg(a.tau_seed + q)),
                           a.eps * a.qtail[(int64_t)q * (L + 1) + l + 1], sh.qterm);
@@ -1311,10 +1311,10 @@ constexpr size_t verify_tc_smem = 1024 + Ring<FP8, 1>::BYTES + sizeof(Shared);
 static_assert(verify_tc_smem<false> <= 113 * 1024 && verify_tc_smem<true> <= 113 * 1024,
               "two CTAs per SM (228 KB, 1 KB of it reserved per CTA)");
 
-int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st) {
+int launch_verify_tc(const VerifyTCArgs& a, bool large, cudaStream_t st) {
   static PerDeviceOnce once;
   using Kernel = void (*)(VerifyTCArgs);
-  // [format][some k above kChainK][panel rows of 128, 64 or 32 bytes at most]
+  // [format][unsorted slots above kChainK][panel rows of 128, 64 or 32 bytes at most]
   static const Kernel kernels[2][2][3] = {
       {{verify_tc_kernel<false, false, 1>, verify_tc_kernel<false, false, 2>,
         verify_tc_kernel<false, false, 4>},
@@ -1352,7 +1352,7 @@ int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st) {
   // persistent CTA that cannot be resident yet starts later and finds the
   // queue drained, so over-provisioning is harmless.
   const int rb = a.max_w * (a.fp8 ? 1 : 2);
-  const Kernel kern = kernels[a.fp8 ? 1 : 0][a.k_max > kChainK ? 1 : 0][rb >= 128 ? 0 : rb == 64 ? 1 : 2];
+  const Kernel kern = kernels[a.fp8 ? 1 : 0][large ? 1 : 0][rb >= 128 ? 0 : rb == 64 ? 1 : 2];
   kern<<<sms * 2, NT, smem, st>>>(a);
   PANO_CUDA(cudaGetLastError());
   return PANO_OK;

@@ -59,6 +59,7 @@ int launch_pack_fp8(const float* xt, const float* rows, const int64_t* perm, int
                     int64_t nchunks, int d, int L, const int32_t* level_off, const float* mu,
                     double c_trans, uint8_t* slices, float* tails, float* xn2, float* ex,
                     float* xscale, int32_t* ids, cudaStream_t st);
-int launch_verify_tc(const VerifyTCArgs& a, cudaStream_t st);
+// large: the slots of queries with k > kChainK are unsorted.
+int launch_verify_tc(const VerifyTCArgs& a, bool large, cudaStream_t st);
 
 }  // namespace pano
