@@ -185,41 +185,29 @@ __global__ void __launch_bounds__(256) pack_fp32_kernel(
     int64_t slot = g * CH + i;
     bool valid = pb[i] >= 0;
     const float* x = xblk + (int64_t)i * d;
-    RowBounds rb;
-    for (int l = L - 1; l >= 0; --l) {
-      Acc2 e{0.f, 0.f};
-      if (valid)
-        for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) acc2_sq(e, x[j]);
-      rb.level(l, warp_acc2_f64(e, level_off[l], level_off[l + 1],
-                                [&](int j) { return (double)x[j] * x[j]; }));
-    }
-    Acc2 dev{0.f, 0.f};  // ||x - mu~||
     const float* r = rows + (lc * CH + i) * (int64_t)d;  // rows of this block
-    if (valid)
-      for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
-    const double de = warp_acc2_f64(dev, 0, d, [&](int j) {
-      const double v = (double)r[j] - (double)mu[j];
-      return v * v;
-    });
+    const RowBounds rb = row_bounds(
+        d, L, level_off, c_trans, valid, [&](int j) { return x[j]; }, [](int) { return 0.0; },
+        [&](int j) { return (double)r[j] - (double)mu[j]; }, [](Acc2&, int, float) {},
+        [&](Acc2& a, int j) { acc2_sqdiff(a, r[j], mu[j]); });
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int l = lane + 32 * u;
       if (l >= L) continue;
-      const float t = rb.tail_norm(u);
+      const float t = rb.tail[u];
       tails[(g * (L + 1) + l) * CH + i] = t;
       if (l > 0) sl[(int64_t)tail_row(l - 1) * CH + i] = t;
     }
     if (lane == 0) {
-      const float exv = valid ? __double2float_ru(c_trans * sqrt(de) * (1.0 + 2e-9)) : 0.f;
       const int32_t id = valid ? (int32_t)pb[i] : -1;
       tails[(g * (L + 1) + L) * CH + i] = 0.f;
       sl[(int64_t)tail_row(L - 1) * CH + i] = 0.f;
-      xn2[slot] = (float)rb.energy;
-      ex[slot] = exv;
+      xn2[slot] = rb.xn2;
+      ex[slot] = rb.ex;
       ids[slot] = id;
       const int64_t r0 = tail_row(0);  // level 0's extra rows
-      sl[(r0 + 1) * CH + i] = (float)rb.energy;
-      sl[(r0 + 2) * CH + i] = exv;
+      sl[(r0 + 1) * CH + i] = rb.xn2;
+      sl[(r0 + 2) * CH + i] = rb.ex;
       sl[(r0 + 3) * CH + i] = __int_as_float(id);
     }
   }

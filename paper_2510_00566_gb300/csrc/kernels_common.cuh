@@ -337,48 +337,129 @@ __device__ __forceinline__ void acc2_sqdiff(Acc2& a, float x, float y) {
   a.c = __fmaf_rn(2.f * h, e, a.c);
 }
 
-__device__ __forceinline__ double acc2_f64(Acc2 a) { return (double)a.s + (double)a.c; }
-
-// The warp's total of a sum as FP64.  A sum that left FP32's range (elements
-// above 1.8e19) is formed again in FP64, from term(j) over j = lo .. hi - 1.
+// The warp's total as FP64, of the squares of value(j), j = lo .. hi - 1.  *ok is
+// cleared where it may be off by more than the bound above and 2^-40: terms
+// beyond FP32's range (elements above 1.8e19), or a total so small that the
+// underflow of squares counts (2^-149 a term; not where all are zeros).
 template <class F>
-__device__ __forceinline__ double warp_acc2_f64(Acc2 a, int lo, int hi, F term) {
-  const double s = acc2_f64(warp_sum_acc2(a));
-  if (fabs(s) < INFINITY) return s;  // (the same in every lane)
-  double t = 0.0;
+__device__ __forceinline__ double warp_acc2_f64(Acc2 a, int lo, int hi, F value, bool* ok) {
+  a = warp_sum_acc2(a);
+  if (!(a.s > 0x1p-90f && a.s < INFINITY)) {  // (the same in every lane)
+    bool nonzero = false;
 #pragma unroll 1
-  for (int j = lo + (int)(threadIdx.x & 31); j < hi; j += 32) t += term(j);
-#pragma unroll 1
-  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-  return t;
+    for (int j = lo + (int)(threadIdx.x & 31); j < hi; j += 32) nonzero |= value(j) != 0.f;
+    if (__any_sync(0xffffffffu, nonzero)) *ok = false;
+  }
+  return (double)a.s + (double)a.c;
 }
-
-// What a packed row's bounds are made of, by one warp: the level energies of
-// the stored vector summed from the last level backwards give the rounded-up
-// tail norms; qerr (the squared storage error) and dev (|x - mu~|^2) give e_x.
-// The sums are compensated FP32 (2^-30 of a sum of non-negative terms at d <=
-// 8192, kept in FP64 from there on), far below the one rounding to FP32 that
-// every result takes: FP64 arithmetic per element was most of the packers'
-// time (a warp's FP64 instruction takes 16 cycles; 500k x 384 BF16 rows: 11.3
-// ms, now 3.0).
-struct RowBounds {
-  double tail[2] = {0.0, 0.0};  // energies from level lane (and lane + 32) on
-  double energy = 0.0;          // of the whole row
-  __device__ __forceinline__ void level(int l, double e) {
-    energy += e;
-    if (l == (int)(threadIdx.x & 31)) tail[0] = energy;
-    if (l == (int)(threadIdx.x & 31) + 32) tail[1] = energy;
-  }
-  // rounded-up sqrt of the energy from this lane's level on (u = 0, 1)
-  __device__ __forceinline__ float tail_norm(int u) const {
-    return __double2float_ru(sqrt(tail[u] * (1.0 + 2e-9)));
-  }
-};
 
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   return v;
+}
+
+// Whether the FP64 value v (normal in FP32) rounds to the same FP32 number, up
+// (NEAREST false) or to nearest, wherever in v (1 -+ r 2^-53) it lies: the 29 bits
+// below FP32's last one stay that far from where the rounding turns.
+template <bool NEAREST>
+__device__ __forceinline__ bool rounds_alike(double v, uint32_t r) {
+  const uint32_t turn = NEAREST ? 1u << 28 : 0u;
+  const uint32_t at = ((uint32_t)__double2loint(v) + turn) & 0x1fffffffu;
+  return at - r < 0x20000000u - 2 * r;
+}
+
+// The bounds of a packed row, by one warp: rounded-up tail norms (of the stored
+// vector, from level `lane` and `lane + 32` on), |x^|^2 and e_x, a bound on the
+// stored vector's distance to the exact transform.
+struct RowBounds {
+  float tail[2], xn2, ex;
+};
+
+// stored(j): the stored element; err(j), dev(j): the storage error and (x - mu~)_j
+// in FP64; add_err(acc, j, stored(j)), add_dev(acc, j): the addition of their
+// squares.
+//
+// All results are those of FP64 sums, rounded once to FP32, but the sums are
+// compensated FP32: FP64 arithmetic per element was most of the packers' time
+// (a warp's FP64 instruction takes 16 cycles; 500k x 384 BF16 rows: 11.3 ms,
+// 3.0 so).  Where a sum's error (a few 1e-12 of it) could move one of the
+// row's results to another FP32 number, the row is summed again in FP64.
+template <class Stored, class Err, class Dev, class AddErr, class AddDev>
+__device__ __forceinline__ RowBounds row_bounds(int d, int L, const int32_t* __restrict__ level_off,
+                                                double c_trans, bool valid, Stored stored, Err err,
+                                                Dev dev, AddErr add_err, AddDev add_dev) {
+  const int lane = threadIdx.x & 31;
+  RowBounds out{{0.f, 0.f}, 0.f, 0.f};
+  if (!valid) return out;
+  constexpr double kUp = 1.0 + 1e-12, kUpE = 1.0 + 1e-9;
+  // error of a sum of n terms in units of 2^-53: the bound of Acc2 with a third
+  // rounding per term (acc2_sqdiff's) and no level additions (they are in
+  // FP64), small terms (2^-40 = 2^13 units), FP64 roundings
+  auto error = [](int n) {
+    const uint32_t m = (uint32_t)(n + 31) / 32;
+    return (4 * m + 16) * (m + 8) * 32 + 8192 + 256;
+  };
+  double tail[2] = {0.0, 0.0}, energy = 0.0;
+  bool ok = true;
+  Acc2 qa{0.f, 0.f}, da{0.f, 0.f};
+  int widest = 0;
+  for (int l = L - 1; l >= 0; --l) {
+    const int lo = level_off[l], hi = level_off[l + 1];
+    Acc2 e{0.f, 0.f};
+    for (int j = lo + lane; j < hi; j += 32) {
+      const float v = stored(j);
+      acc2_sq(e, v);
+      add_err(qa, j, v);
+    }
+    widest = max(widest, hi - lo);
+    energy += warp_acc2_f64(e, lo, hi, stored, &ok);
+    if (l == lane) tail[0] = energy;
+    if (l == lane + 32) tail[1] = energy;
+  }
+  for (int j = lane; j < d; j += 32) add_dev(da, j);
+  const double qe = warp_acc2_f64(qa, 0, d, err, &ok), de = warp_acc2_f64(da, 0, d, dev, &ok);
+  // (lanes 0 and 1 take a root each: FP64 roots are long)
+  const double root = sqrt(lane == 0 ? qe : de);
+  const double e =
+      (__shfl_sync(0xffffffffu, root, 0) + c_trans * __shfl_sync(0xffffffffu, root, 1)) * kUpE;
+  const uint32_t r = error(widest);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (32 * u >= L) break;
+    const double t = sqrt(tail[u] * kUp);
+    out.tail[u] = __double2float_ru(t);
+    if (t > 0.0) ok &= rounds_alike<false>(t, r);
+  }
+  out.xn2 = (float)energy;
+  out.ex = __double2float_ru(e);
+  if (energy > 0.0) ok &= rounds_alike<true>(energy, r);
+  if (e > 0.0) ok &= rounds_alike<false>(e, error(d));
+  if (__all_sync(0xffffffffu, ok)) return out;
+  double q2 = 0.0, d2 = 0.0;
+  energy = 0.0;
+#pragma unroll 1
+  for (int l = L - 1; l >= 0; --l) {
+    double s = 0.0;
+#pragma unroll 1
+    for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) {
+      const double v = stored(j), q = err(j);
+      s += v * v;
+      q2 += q * q;
+    }
+    energy += warp_sum_f64(s);
+    const float t = __double2float_ru(sqrt(energy * kUp));
+    if (l == lane) out.tail[0] = t;
+    if (l == lane + 32) out.tail[1] = t;
+  }
+#pragma unroll 1
+  for (int j = lane; j < d; j += 32) {
+    const double v = dev(j);
+    d2 += v * v;
+  }
+  out.xn2 = (float)energy;
+  out.ex = __double2float_ru((sqrt(warp_sum_f64(q2)) + c_trans * sqrt(warp_sum_f64(d2))) * kUpE);
+  return out;
 }
 
 }  // namespace pano

@@ -91,43 +91,21 @@ __global__ void __launch_bounds__(256) pack_bf16_kernel(
     const bool valid = pb[i] >= 0;
     const float* x = xblk + (int64_t)i * d;
     auto stored = [](float v) { return __bfloat162float(__float2bfloat16_rn(v)); };
-    RowBounds rb;
-    Acc2 qerr{0.f, 0.f};
-    for (int l = L - 1; l >= 0; --l) {
-      Acc2 e{0.f, 0.f};
-      if (valid)
-        for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) {
-          const float xf = x[j], xh = stored(xf);
-          acc2_sq(e, xh);
-          acc2_sq(qerr, __fsub_rn(xh, xf));  // (exact: xh is within a factor 2 of xf)
-        }
-      rb.level(l, warp_acc2_f64(e, level_off[l], level_off[l + 1], [&](int j) {
-                 const double v = stored(x[j]);
-                 return v * v;
-               }));
-    }
-    Acc2 dev{0.f, 0.f};
     const float* r = rows + (lc * CH + i) * (int64_t)d;
-    if (valid)
-      for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
-    // lanes 0 and 1 take a root each (FP64 roots are long)
-    const double qe = warp_acc2_f64(qerr, 0, d, [&](int j) {
-      const double v = (double)stored(x[j]) - (double)x[j];
-      return v * v;
-    });
-    const double de = warp_acc2_f64(dev, 0, d, [&](int j) {
-      const double v = (double)r[j] - (double)mu[j];
-      return v * v;
-    });
-    const double root = sqrt(lane == 0 ? qe : de);
-    const double dev_root = __shfl_sync(0xffffffffu, root, 1);
+    const RowBounds rb = row_bounds(
+        d, L, level_off, c_trans, valid, [&](int j) { return stored(x[j]); },
+        [&](int j) { return (double)stored(x[j]) - (double)x[j]; },
+        [&](int j) { return (double)r[j] - (double)mu[j]; },
+        // (exact: xh is within a factor 2 of x[j])
+        [&](Acc2& a, int j, float xh) { acc2_sq(a, __fsub_rn(xh, x[j])); },
+        [&](Acc2& a, int j) { acc2_sqdiff(a, r[j], mu[j]); });
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail_norm(u);
+      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail[u];
     if (lane == 0) {
       tails[(g * (L + 1) + L) * CH + i] = 0.f;
-      xn2[slot] = (float)rb.energy;
-      ex[slot] = valid ? __double2float_ru((root + c_trans * dev_root) * (1.0 + 2e-9)) : 0.f;
+      xn2[slot] = rb.xn2;
+      ex[slot] = rb.ex;
       ids[slot] = valid ? (int32_t)pb[i] : -1;
     }
   }
@@ -192,43 +170,20 @@ __global__ void __launch_bounds__(256) pack_fp8_kernel(
     const float* x = xblk + (int64_t)i * d;
     const float sc = s_scale[i], inv = s_inv[i];
     auto stored = [&](float v) { return tc::e4m3_to_f32(tc::f32_to_e4m3(v * inv)) * sc; };
-    RowBounds rb;
-    Acc2 qerr{0.f, 0.f};
-    for (int l = L - 1; l >= 0; --l) {
-      Acc2 e{0.f, 0.f};
-      if (valid)
-        for (int j = level_off[l] + lane; j < level_off[l + 1]; j += 32) {
-          const float xf = x[j], xh = stored(xf);
-          acc2_sq(e, xh);
-          acc2_sqdiff(qerr, xh, xf);
-        }
-      rb.level(l, warp_acc2_f64(e, level_off[l], level_off[l + 1], [&](int j) {
-                 const double v = stored(x[j]);
-                 return v * v;
-               }));
-    }
-    Acc2 dev{0.f, 0.f};
     const float* r = rows + (lc * CH + i) * (int64_t)d;
-    if (valid)
-      for (int j = lane; j < d; j += 32) acc2_sqdiff(dev, r[j], mu[j]);
-    // lanes 0 and 1 take a root each (FP64 roots are long)
-    const double qe = warp_acc2_f64(qerr, 0, d, [&](int j) {
-      const double v = (double)stored(x[j]) - (double)x[j];
-      return v * v;
-    });
-    const double de = warp_acc2_f64(dev, 0, d, [&](int j) {
-      const double v = (double)r[j] - (double)mu[j];
-      return v * v;
-    });
-    const double root = sqrt(lane == 0 ? qe : de);
-    const double dev_root = __shfl_sync(0xffffffffu, root, 1);
+    const RowBounds rb = row_bounds(
+        d, L, level_off, c_trans, valid, [&](int j) { return stored(x[j]); },
+        [&](int j) { return (double)stored(x[j]) - (double)x[j]; },
+        [&](int j) { return (double)r[j] - (double)mu[j]; },
+        [&](Acc2& a, int j, float xh) { acc2_sqdiff(a, xh, x[j]); },
+        [&](Acc2& a, int j) { acc2_sqdiff(a, r[j], mu[j]); });
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail_norm(u);
+      if (lane + 32 * u < L) tails[(g * (L + 1) + lane + 32 * u) * CH + i] = rb.tail[u];
     if (lane == 0) {
       tails[(g * (L + 1) + L) * CH + i] = 0.f;
-      xn2[slot] = (float)rb.energy;
-      ex[slot] = valid ? __double2float_ru((root + c_trans * dev_root) * (1.0 + 2e-9)) : 0.f;
+      xn2[slot] = rb.xn2;
+      ex[slot] = rb.ex;
       xscale[slot] = sc;
       ids[slot] = valid ? (int32_t)pb[i] : -1;
     }
