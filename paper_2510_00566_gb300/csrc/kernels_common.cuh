@@ -353,6 +353,21 @@ __device__ __forceinline__ double warp_acc2_f64(Acc2 a, int lo, int hi, F value,
   return (double)a.s + (double)a.c;
 }
 
+// The root of the sum held by a, rounded to nearest, as FP64 would give it from
+// a sum off by at most rel; NaN where that cannot be told from a.
+__device__ __forceinline__ float sqrt_rn_acc2(Acc2 a, float rel) {
+  float lo;
+  const float hi = two_sum(a.s, a.c, lo);
+  if (hi == 0.f) return 0.f;
+  if (!(hi > 0x1p-80f && hi < 0x1p120f)) return NAN;
+  // the exact root is r + delta up to 2^-44 of r
+  const float r = __fsqrt_rn(hi);
+  const float delta = __fdividef(__fadd_rn(__fmaf_rn(-r, r, hi), lo), 2.f * r);
+  const float slack = r * (0.5f * rel + 0x1p-43f);
+  const float up = __fadd_rn(r, delta + slack), down = __fadd_rn(r, delta - slack);
+  return up == down ? up : NAN;
+}
+
 __device__ __forceinline__ double warp_sum_f64(double v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);

@@ -324,6 +324,7 @@ struct PqArgs {
   int d, M, dsub, L, ML, b, k_max, prune, collect;
   int slab;    // candidates per slab of one (query, list) pair, PQ_S at most
   float lo;    // (1 - gamma) factor of the lower bound, rounded down
+  float srel;  // error of a level's compensated sums and of their tail sums
   float erel;  // relative allowance for the roundings of s_q, s_x and |s_q - s_x|
   float eps;   // Eq. 4 (1 = the exact, margined test)
 };
@@ -577,8 +578,15 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
   // block builds level 0's table (the first slab needs it when it is large)
   for (int l = warp; l < L; l += PQ_NT / 32) {
     Acc2 s{0.f, 0.f};
-    for (int j = lane; j < a.b; j += 32) acc2_sq(s, r[l * a.b + j]);
+    uint32_t bits = 0;
+    for (int j = lane; j < a.b; j += 32) {
+      acc2_sq(s, r[l * a.b + j]);
+      bits |= __float_as_uint(r[l * a.b + j]);
+    }
     s = warp_sum_acc2(s);
+    // (squares that underflow, or leave FP32's range: NaN from here on)
+    const bool zero = __reduce_or_sync(0xffffffffu, bits) << 1 == 0;
+    if (!zero && !(s.s > 0x1p-90f && s.s < INFINITY)) s.s = NAN;
     if (lane == 0) eq[l] = s;
   }
   int lut_level = -1;  // the level whose table `lut` holds (uniform)
@@ -589,19 +597,20 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
     n_lut = 1;
   }
   __syncthreads();
-  // tail after level l: one lane per level; its root is within 1.5 u
+  // tail after level l: one lane per level, its root rounded to nearest as from
+  // an FP64 sum; where the compensated sum does not settle it, from an FP64 sum
   if (warp == 0)
     for (int l = lane; l < L; l += 32) {
       Acc2 tail{0.f, 0.f};
       for (int l2 = L - 1; l2 > l; --l2) acc2_add(tail, eq[l2]);
-      const float e = __fadd_rn(tail.s, tail.c);
-      if (e < INFINITY) {
-        sq[l] = __fsqrt_rn(e);
-      } else {  // beyond FP32's range: the sum again in FP64
+      float root = sqrt_rn_acc2(tail, a.srel);
+      if (!(root >= 0.f)) {
         double t = 0.0;
+#pragma unroll 1
         for (int j = (l + 1) * a.b; j < d; ++j) t += (double)r[j] * r[j];
-        sq[l] = (float)sqrt(t);
+        root = (float)sqrt(t);
       }
+      sq[l] = root;
     }
   __syncthreads();
 
@@ -1255,9 +1264,10 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     float lo32 = (float)lo;
     if ((double)lo32 > lo) lo32 = std::nextafter(lo32, 0.f);
     a.lo = lo32;
-    // s_q: a compensated sum and its root rounded (1.5 u), s_x: an FP64 sum
-    // rounded to FP32 (u), |s_q - s_x| and the allowance itself (u each): 8u of
-    // (s_q + s_x) covers them with margin.
+    // s_q, s_x: FP64 sums rounded to FP32 (u each), |s_q - s_x| and the
+    // allowance itself (u each): 8u of (s_q + s_x) covers them with margin.
+    const double sm = (a.b + 31) / 32;
+    a.srel = (float)((2 * sm + 2 * L + 12) * (sm + L + 6) * 0x1p-48 * 1.01);
     a.erel = (float)(8.0 * kU32);
     a.eps = (epsilon > 0.f && epsilon < 1.f) ? epsilon : 1.f;
 
