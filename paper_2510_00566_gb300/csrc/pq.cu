@@ -3,7 +3,7 @@
 //
 // Search: one thread block per (query, probed list) pair.  The block forms
 // the query residual r = q~ - c~ in shared memory and its level tail
-// energies, then walks the list in slabs of a.slab candidates.  A
+// energies, then walks the list in slabs of PQ_S candidates.  A
 // level's subvector terms e_m = ||r_m - C_m[code_m]||^2 come from a table of
 // the 256 terms of each of the level's subquantisers in shared memory (the
 // paper's per-level look-up tables) while many candidates are live, and
@@ -39,7 +39,7 @@ namespace {
 
 constexpr int PQ_KSUB = 256;     // codewords per subquantiser (8-bit codes)
 constexpr int PQ_B = 256;        // vector slots per layout block
-constexpr int PQ_S = 2048;       // candidates per slab at most of one (query, list) pair
+constexpr int PQ_S = 2048;       // candidates per slab of one (query, list) pair
 constexpr int PQ_NT = 256;       // threads of the verify kernel
 constexpr int PQ_MAXML = 64;     // subquantisers per level
 constexpr int PQ_MAXDSUB = 32;   // coordinates per subvector
@@ -322,7 +322,6 @@ struct PqArgs {
   unsigned long long* topk;
   unsigned long long* stats;
   int d, M, dsub, L, ML, b, k_max, prune, collect;
-  int slab;    // candidates per slab of one (query, list) pair, PQ_S at most
   float lo;    // (1 - gamma) factor of the lower bound, rounded down
   float srel;  // error of a level's compensated sums and of their tail sums
   float erel;  // relative allowance for the roundings of s_q, s_x and |s_q - s_x|
@@ -330,7 +329,7 @@ struct PqArgs {
 };
 
 // Bytes of dynamic shared memory of the verify kernel.
-size_t pq_verify_smem(int d, int L, int ML, int slab) {
+size_t pq_verify_smem(int d, int L, int ML) {
   size_t o = 0;
   auto take = [&](size_t bytes) {
     o = (o + 15) & ~(size_t)15;
@@ -340,8 +339,8 @@ size_t pq_verify_smem(int d, int L, int ML, int slab) {
   take((size_t)L * 8);                 // level energies (compensated FP32)
   take((size_t)L * 4);                 // s_q per level
   take((size_t)ML * PQ_KSUB * 4);      // level table
-  take((size_t)2 * slab * 4);          // partial distances (two lists)
-  take((size_t)2 * slab * 2);          // live candidates (two lists)
+  take((size_t)2 * PQ_S * 4);          // partial distances (two lists)
+  take((size_t)2 * PQ_S * 2);          // live candidates (two lists)
   take(64);                            // counters, threshold
   return o;
 }
@@ -523,9 +522,12 @@ __device__ __forceinline__ void level_sum4(const uint32_t* __restrict__ cp, int 
   }
 }
 
-__global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
+// BPS: blocks per SM (four where shared memory allows them; 80 registers at
+// three spill nothing).
+template <int BPS>
+__global__ void __launch_bounds__(PQ_NT, BPS) pq_verify_kernel(const PqArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int d = a.d, L = a.L, ML = a.ML, M = a.M, dsub = a.dsub, slab = a.slab;
+  const int d = a.d, L = a.L, ML = a.ML, M = a.M, dsub = a.dsub;
   size_t o = 0;
   auto carve = [&](size_t bytes) {
     o = (o + 15) & ~(size_t)15;
@@ -537,8 +539,8 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
   Acc2* eq = (Acc2*)carve((size_t)L * 8);
   float* sq = (float*)carve((size_t)L * 4);
   float* lut = (float*)carve((size_t)ML * PQ_KSUB * 4);
-  float* pacc = (float*)carve((size_t)2 * slab * 4);
-  uint16_t* live = (uint16_t*)carve((size_t)2 * slab * 2);
+  float* pacc = (float*)carve((size_t)2 * PQ_S * 4);
+  uint16_t* live = (uint16_t*)carve((size_t)2 * PQ_S * 2);
   int* ctr = (int*)carve(64);  // [0] survivors of the level, [2] threshold bits, [3] k,
                                // [8..15] four 64-bit section clocks
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -591,7 +593,7 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
   }
   int lut_level = -1;  // the level whose table `lut` holds (uniform)
   unsigned long long n_lut = 0;
-  if (min(slab, nc) >= PQ_LUT_MIN) {
+  if (min(PQ_S, nc) >= PQ_LUT_MIN) {
     build_table(lut, r, a.codebook, 0, ML, dsub);
     lut_level = 0;
     n_lut = 1;
@@ -617,8 +619,8 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
   lap(0);
   // counters (every thread keeps its own; summed at the end when collecting)
   unsigned long long n_dims = 0, n_lv = 0, n_full = 0;
-  for (int s0 = 0; s0 < nc; s0 += slab) {
-    const int ns = min(slab, nc - s0);
+  for (int s0 = 0; s0 < nc; s0 += PQ_S) {
+    const int ns = min(PQ_S, nc - s0);
     int nl = ns, cur = 0;
     for (int l = 0; l < L && nl > 0; ++l) {
       const bool last = l == L - 1;
@@ -628,8 +630,8 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
         // tables), stopping at the first level whose test fails; no block
         // barrier per level
         for (int i = tid; i < nl; i += PQ_NT) {
-          const int cand = live[cur * slab + i];
-          float P = pacc[cur * slab + i];
+          const int cand = live[cur * PQ_S + i];
+          float P = pacc[cur * PQ_S + i];
           const int g = s0 + cand;
           const int64_t blk = blk0 + g / PQ_B;
           const int ln = g % PQ_B;
@@ -713,14 +715,14 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
             }
           }
         } else if (i < nunits) {
-          cand0 = live[cur * slab + i];
+          cand0 = live[cur * PQ_S + i];
           const int g = s0 + cand0;
           const int64_t blk = blk0 + g / PQ_B;
           const int ln = g % PQ_B;
           const uint8_t* cp = a.codes + (blk * M + (int64_t)l * ML) * PQ_B + ln;
           const float S = use_lut ? level_sum1<true>(cp, ML, l * ML, lut, r, a.codebook, dsub)
                                   : level_sum_direct(cp, ML, l * ML, r, a.codebook, dsub);
-          const float P = __fadd_rn(pacc[cur * slab + i], S);
+          const float P = __fadd_rn(pacc[cur * PQ_S + i], S);
           Pv[0] = P;
           if (last) {
             const unsigned long long key = make_key(P, a.ids[blk * PQ_B + ln]);
@@ -739,8 +741,8 @@ __global__ void __launch_bounds__(PQ_NT, 4) pq_verify_kernel(const PqArgs a) {
             base = __shfl_sync(0xffffffffu, base, 0);
             if (keep[c]) {
               const int at = base + __popc(ball & ((1u << lane) - 1));
-              live[nxt * slab + at] = (uint16_t)(cand0 + c);
-              pacc[nxt * slab + at] = Pv[c];
+              live[nxt * PQ_S + at] = (uint16_t)(cand0 + c);
+              pacc[nxt * PQ_S + at] = Pv[c];
             }
           }
         }
@@ -1277,14 +1279,13 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     pq_seed_kernel<<<(unsigned)nq, 256, ssm, st>>>(a, probes, nprobe);
     PANO_CUDA(cudaGetLastError());
     mark(3);
-    // lists of up to about 1,024 vectors fill one slab of half the size, and
-    // four blocks share an SM (250k x 960 on 256 lists, 4,096 queries: 3.87 ms
-    // with three, now 3.5)
-    a.slab = I.n <= (int64_t)1100 * nlist ? PQ_S / 2 : PQ_S;
-    const size_t vsm = pq_verify_smem(d, L, ML, a.slab);
-    PANO_CUDA(cudaFuncSetAttribute(pq_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)vsm));
-    pq_verify_kernel<<<(unsigned)npairs, PQ_NT, vsm, st>>>(a);
+    const size_t vsm = pq_verify_smem(d, L, ML);
+    int per_sm = 0;
+    PANO_CUDA(cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, I.device));
+    // (1 KB of a block's shared memory is the system's)
+    auto verify = 4 * (vsm + 1024) <= (size_t)per_sm ? pq_verify_kernel<4> : pq_verify_kernel<3>;
+    PANO_CUDA(cudaFuncSetAttribute(verify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vsm));
+    verify<<<(unsigned)npairs, PQ_NT, vsm, st>>>(a);
     PANO_CUDA(cudaGetLastError());
     mark(4);
     pq_decode_kernel<<<(unsigned)((nq * k_max + 255) / 256), 256, 0, st>>>(topk, nq * k_max, out_ids,
