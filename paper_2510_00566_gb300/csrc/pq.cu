@@ -1225,7 +1225,7 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
     PANO_CUDA(gemm_nt(kStore, (int)nq, d, d, queries, d, I.mu32.as<float>(), I.T32.as<float>(),
                       d, qt, d, nullptr, nullptr, st));
     mark(1);
-    int rc = probe_only(ip, queries, nq, nprobe, probes, st, false);
+    int rc = probe_only(ip, queries, nq, nprobe, probes, st, (int*)(stats + 15));
     if (rc) return rc;
     mark(2);
     const unsigned pg = (unsigned)((npairs + 255) / 256);
@@ -1319,6 +1319,8 @@ int search_pq(const pano_index* ip, const float* queries, int64_t nq, const int3
       // block clocks: prologue, level-0 tables, level-0 scan, deeper levels
       for (int i = 0; i < 4; ++i) S.section_cycles[i] = (int64_t)hs[8 + i];
     }
+    // (the last word is the probe's error word)
+    if ((int)hs[15] & kErrTimeout) return fail(PANO_ETIMEOUT, "a device-side wait timed out");
     return PANO_OK;
   };
   int rc = body();

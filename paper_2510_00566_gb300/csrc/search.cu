@@ -2160,7 +2160,7 @@ int status_of_device_error(int word) {
 }
 
 int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t nprobe,
-               int32_t* out, cudaStream_t st, bool sync) {
+               int32_t* out, cudaStream_t st, int* err_word) {
   PANO_CHECK(ip, PANO_EINVAL, "null index");
   const pano_index& I = *ip;
   PANO_CHECK(nprobe >= 1 && nprobe <= I.nlist, PANO_EINVAL, "nprobe must be in [1, nlist]");
@@ -2183,9 +2183,9 @@ int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t n
   float* pd = (float*)(W + o_pd);
   float* qn2 = (float*)(W + o_qn);
   int32_t* npq = (int32_t*)(W + o_np);
-  int* err = (int*)(W + o_err);
+  int* err = err_word ? err_word : (int*)(W + o_err);
   auto body = [&]() -> int {
-    PANO_CUDA(cudaMemsetAsync(err, 0, 16, st));
+    if (!err_word) PANO_CUDA(cudaMemsetAsync(err, 0, 16, st));
     prep_kernel<<<(unsigned)((nq + 255) / 256), 256, 0, st>>>(nq, nullptr, nprobe, nlist, nullptr,
                                                               0, 1, npq, npq + nq, err);
     row_sqnorm_kernel<<<(unsigned)((nq + 7) / 8), 256, 0, st>>>(queries, nq, d, qn2);
@@ -2205,7 +2205,11 @@ int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t n
     probe_select_kernel<<<(unsigned)nq, NT, psm, st>>>(pd, nlist, queries, I.cent.as<float>(), d,
                                                        qn2, I.cmax, gerr, npq, nprobe, out, err, 1);
     PANO_CUDA(cudaGetLastError());
-    if (sync) PANO_CUDA(cudaStreamSynchronize(st));
+    if (err_word) return PANO_OK;
+    int herr = 0;
+    PANO_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    PANO_CUDA(cudaStreamSynchronize(st));
+    if (herr & kErrTimeout) return fail(PANO_ETIMEOUT, "a device-side wait timed out");
     return PANO_OK;
   };
   int rc = body();

@@ -16,8 +16,10 @@ int search_workspace_bytes(const pano_index* ip, int64_t nq, int32_t stride, int
 // Status code of a device error word (kErrTimeout -> PANO_ETIMEOUT,
 // kErrBadInput -> PANO_EINVAL, otherwise PANO_OK).
 int status_of_device_error(int word);
+// err: a zeroed device error word that the caller reads after the stream has
+// passed (the call does not wait then); null: it waits and checks its own.
 int probe_only(const pano_index* ip, const float* queries, int64_t nq, int32_t nprobe,
-               int32_t* out, cudaStream_t st, bool sync = true);
+               int32_t* out, cudaStream_t st, int* err = nullptr);
 const pano_search_stats& last_stats();
 pano_search_stats& stats_slot();  // the calling thread's last-call statistics
 int transform_queries(const pano_index& I, const float* queries, int64_t nq, float* qt,
