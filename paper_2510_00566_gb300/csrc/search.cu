@@ -1712,7 +1712,9 @@ struct SearchLayout {
   size_t total = 0;
 };
 
-int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLayout* out) {
+// whole: FP32 segments of full length whatever the batch.
+int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLayout* out,
+                bool whole = false) {
   SearchLayout& y = *out;
   const int d = I.d, L = I.L, nlist = I.nlist;
   const bool tcpath = I.precision != PANO_FP32;
@@ -1726,7 +1728,7 @@ int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLa
   // the mean size)
   const int64_t mean_seg = I.n_chunks / ((int64_t)nlist * SEG_CHUNKS) + 1;
   const int64_t groups = (nq + QBA - 1) / QBA + std::min<int64_t>(nq, nlist - 1);
-  y.seg = tcpath ? TC_SEG : seg_chunks(groups * mean_seg);
+  y.seg = tcpath ? TC_SEG : whole ? SEG_CHUNKS : seg_chunks(groups * mean_seg);
   const int SEG = y.seg;
   // work-item capacity: groups x segments, plus one partial group per list
   int64_t max_seg = 1, tot_seg = 0;
@@ -1809,6 +1811,10 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
   const bool tcpath = I.precision != PANO_FP32;
   SearchLayout lay;
   if (int r = plan_layout(I, nq, stride, k_max, &lay)) return r;
+  // (short segments have more work items: a workspace of fixed size that lacks
+  // the room for them takes full ones)
+  if (ext_ws && lay.total > ext_cap)
+    if (int r = plan_layout(I, nq, stride, k_max, &lay, true)) return r;
   const TileCfg tileA = lay.tileA, tileB = lay.tileB;
   const int bpsA = lay.bpsA, bpsB = lay.bpsB;
   const int QBA = tileA.QB, QBB = tileB.QB;
