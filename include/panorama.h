@@ -163,7 +163,9 @@ typedef struct {
   int32_t chunk;        /* vectors per level-major chunk                     */
   int32_t max_level_width;
   int64_t n_chunks;
-  int64_t device_bytes; /* device memory held by the index                   */
+  int64_t device_bytes; /* device memory held by the index; not counted: up to
+                           1 GiB of search workspace that all indexes of a
+                           device keep together while one of them lives     */
   double eta;           /* ||T~^T T~ - I||_F of the FP32 transform            */
 } pano_index_info;
 

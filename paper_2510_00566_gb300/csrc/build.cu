@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstring>
 #include <numeric>
+#include <unordered_map>
 
 #include "gemm.h"
 #include "internal.h"
@@ -415,15 +416,23 @@ int DevBuf::alloc(size_t n) {
 }
 
 int WsPool::create(int device) {
+  using Held = std::weak_ptr<std::remove_pointer_t<cudaMemPool_t>>;
+  static std::mutex mu;
+  static auto& pools = *new std::unordered_map<int, Held>;  // (outlives every index)
+  std::lock_guard<std::mutex> lock(mu);
+  if ((pool = pools[device].lock())) return PANO_OK;
   cudaMemPoolProps props = {};
   props.allocType = cudaMemAllocationTypePinned;
   props.location.type = cudaMemLocationTypeDevice;
   props.location.id = device;
-  PANO_CUDA(cudaMemPoolCreate(&pool, &props));
+  cudaMemPool_t made = nullptr;
+  PANO_CUDA(cudaMemPoolCreate(&made, &props));
+  pool.reset(made, [](cudaMemPool_t p) { cudaMemPoolDestroy(p); });
   uint64_t keep = kKeep;
   int off = 0;
-  PANO_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-  PANO_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off));
+  PANO_CUDA(cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep));
+  PANO_CUDA(cudaMemPoolSetAttribute(made, cudaMemPoolReuseAllowInternalDependencies, &off));
+  pools[device] = pool;
   return PANO_OK;
 }
 
@@ -432,7 +441,7 @@ cudaError_t WsPool::alloc(void** p, size_t bytes, cudaStream_t st) const {
   cudaError_t e = cudaStreamIsCapturing(st, &cap);
   if (e != cudaSuccess) return e;
   if (cap != cudaStreamCaptureStatusNone) return cudaMallocAsync(p, bytes, st);
-  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+  return cudaMallocFromPoolAsync(p, bytes, pool.get(), st);
 }
 
 void DevBuf::release() {

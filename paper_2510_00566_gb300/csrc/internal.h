@@ -91,23 +91,18 @@ struct DevBuf {
   DevBuf& operator=(const DevBuf&) = delete;
 };
 
-// Pool of an index's search workspaces.  The default pool gives its memory back
-// at every synchronization, so each synchronous search mapped its workspace
-// anew (0.1 to 0.4 ms); this one keeps up to kKeep bytes and goes with the
-// index.  No dependencies between streams are inserted for the sake of reuse:
-// searches on several streams overlap as before.
+// An index's hold on its device's pool of search workspaces.  The default pool
+// gives its memory back at every synchronization, so each synchronous search
+// mapped its workspace anew (0.1 to 0.4 ms); this one keeps up to kKeep bytes
+// for all indexes of the device together and goes with the last of them.  No
+// dependencies between streams are inserted for the sake of reuse: searches on
+// several streams overlap as before.
 struct WsPool {
   static constexpr uint64_t kKeep = (uint64_t)1 << 30;
-  cudaMemPool_t pool = nullptr;
+  std::shared_ptr<std::remove_pointer_t<cudaMemPool_t>> pool;
   int create(int device);
   // In a stream capture the allocation becomes a graph node of its own pool.
   cudaError_t alloc(void** p, size_t bytes, cudaStream_t st) const;
-  ~WsPool() {
-    if (pool) cudaMemPoolDestroy(pool);
-  }
-  WsPool() = default;
-  WsPool(const WsPool&) = delete;
-  WsPool& operator=(const WsPool&) = delete;
 };
 
 }  // namespace pano
