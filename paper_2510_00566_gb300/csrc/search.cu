@@ -42,9 +42,9 @@ constexpr int SEG_CHUNKS = 32;  // chunks per work-item segment of a large FP32 
 // A small batch takes shorter segments, until there are a few items per SM:
 // 100 queries on one list of 20,000 were 70 items on 152 SMs (295 us, now
 // 103).  `items` counts the batch's (query group, full segment) pairs.
-inline int seg_chunks(int64_t items) {
+inline int seg_chunks(int64_t items, int sms) {
   int seg = SEG_CHUNKS;
-  while (seg > 4 && items < 608) seg /= 2, items *= 2;
+  while (seg > 4 && items < 4 * sms) seg /= 2, items *= 2;
   return seg;
 }
 constexpr int NT = 256;
@@ -617,7 +617,10 @@ __global__ void __launch_bounds__(W * 32) seed_tau_kernel(
 // Zipf-sized lists).
 constexpr int kSeedSub = 16;
 // (fewer queries per group where 16 would leave SMs without one)
-inline int seed_sub_of(int64_t nq) { return nq >= 16 * 304 ? 16 : nq >= 4 * 304 ? 8 : nq >= 304 ? 4 : 2; }
+inline int seed_sub_of(int64_t nq, int sms) {
+  const int64_t per = nq / (2 * sms);  // queries per CTA at two CTAs an SM
+  return per >= 16 ? 16 : per >= 4 ? 8 : per >= 1 ? 4 : 2;
+}
 
 __global__ void __launch_bounds__(kSeedWarps * 32) seed_group_kernel(
     const float* __restrict__ q, int d, const int* __restrict__ soff, int nlist,
@@ -1704,7 +1707,7 @@ thread_local pano_search_stats t_stats;
 // tiles of the FP32 verify phases, the work-item capacities and the carve.
 struct SearchLayout {
   TileCfg tileA{TC_QG, 0, 0, 0}, tileB{TC_QG, 0, 0, 0};
-  int bpsA = 0, bpsB = 0, seg = 0;
+  int bpsA = 0, bpsB = 0, seg = 0, sms = 0;
   int64_t capA = 0, capB = 0;
   size_t o_qt, o_qinfo, o_qtail, o_qn2, o_pd, o_pr, o_npq, o_kq, o_seed, o_cnt, o_fill, o_boff,
       o_ioff, o_tot, o_bucket, o_itA, o_itB, o_topk, o_err, o_stats;
@@ -1717,6 +1720,9 @@ int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLa
                 bool whole = false) {
   SearchLayout& y = *out;
   const int d = I.d, L = I.L, nlist = I.nlist;
+  int sms = 0;
+  PANO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, I.device));
+  y.sms = sms;
   const bool tcpath = I.precision != PANO_FP32;
   if (!tcpath) {
     int r = pick_tile(kTilesA, 3, I.max_w, L, &y.tileA, &y.bpsA);
@@ -1728,7 +1734,7 @@ int plan_layout(const pano_index& I, int64_t nq, int stride, int k_max, SearchLa
   // the mean size)
   const int64_t mean_seg = I.n_chunks / ((int64_t)nlist * SEG_CHUNKS) + 1;
   const int64_t groups = (nq + QBA - 1) / QBA + std::min<int64_t>(nq, nlist - 1);
-  y.seg = tcpath ? TC_SEG : whole ? SEG_CHUNKS : seg_chunks(groups * mean_seg);
+  y.seg = tcpath ? TC_SEG : whole ? SEG_CHUNKS : seg_chunks(groups * mean_seg, sms);
   const int SEG = y.seg;
   // work-item capacity: groups x segments, plus one partial group per list
   int64_t max_seg = 1, tot_seg = 0;
@@ -1818,7 +1824,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
   const TileCfg tileA = lay.tileA, tileB = lay.tileB;
   const int bpsA = lay.bpsA, bpsB = lay.bpsB;
   const int QBA = tileA.QB, QBB = tileB.QB;
-  const int SEG = lay.seg;
+  const int SEG = lay.seg, sms = lay.sms;
   const int64_t capA = lay.capA, capB = lay.capB;
   const size_t o_qt = lay.o_qt, o_qinfo = lay.o_qinfo, o_qtail = lay.o_qtail, o_qn2 = lay.o_qn2,
                o_pd = lay.o_pd, o_pr = lay.o_pr, o_npq = lay.o_npq, o_kq = lay.o_kq,
@@ -1928,7 +1934,7 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
                                                                    nlist, first_rank_b);
     // (the seed groups' scan takes the place of the probe distances)
     int* soff = nlist > 1 ? (int*)P(o_pd) : nullptr;
-    const int seed_sub = seed_sub_of(nq);
+    const int seed_sub = seed_sub_of(nq, sms);
     inv_scan_kernel<<<1, 1024, 0, st>>>(cnt, nlist, I.chunk_off_d.as<int64_t>(), SEG, QBA, QBB,
                                         seed_sub, boff, ioff, soff, tot);
     inv_scatter_kernel<<<(unsigned)((ne + 255) / 256), 256, 0, st>>>(
@@ -1959,8 +1965,9 @@ int search(const pano_index* ip, const float* queries, int64_t nq, const int32_t
           I.list_size_d.as<int32_t>(), I.chunk, I.rows.as<float>(), kq, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
     } else {
-      auto seeds = nq < 152 ? seed_tau_kernel<16> : seed_tau_kernel<kSeedWarps>;
-      seeds<<<(unsigned)nq, (nq < 152 ? 16 : kSeedWarps) * 32, (size_t)d * 4, st>>>(
+      const bool few = nq < sms;
+      auto seeds = few ? seed_tau_kernel<16> : seed_tau_kernel<kSeedWarps>;
+      seeds<<<(unsigned)nq, (few ? 16 : kSeedWarps) * 32, (size_t)d * 4, st>>>(
           queries, d, probes, stride, I.chunk_off_d.as<int64_t>(), I.list_size_d.as<int32_t>(),
           I.chunk, I.rows.as<float>(), kq, one_pass ? nullptr : bucket, seed_slack, tau_seed,
           I.ids.as<int32_t>(), eps < 1.f ? topk : nullptr, k_max);
