@@ -101,18 +101,8 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
 // once all inserts have finished the slots hold the k smallest keys ever
 // inserted, in ascending order.  A slot whose current value is already below
 // the carried key would keep it, so those steps are skipped.
-__device__ __forceinline__ void topk_insert(unsigned long long* slots, int k,
-                                            unsigned long long key) {
-  int j = 0;
-  while (j < k && ld_volatile_u64(slots + j) < key) ++j;
-  for (; j < k; ++j) {
-    unsigned long long old = atomicMin(slots + j, key);
-    if (old == kEmptyKey || old == key) return;  // an equal key is the same pair: kept once
-    key = old > key ? old : key;
-  }
-}
-
-// topk_insert by one thread whose slot reads go out in batches of eight
+//
+// By one thread: its slot reads go out in batches of eight
 // independent loads (one round per eight slots, not one per slot), so that
 // many threads can each insert a key at once and their compare-exchange
 // chains overlap.  A read may be stale: slots only ever decrease, so the
@@ -136,7 +126,7 @@ __device__ __forceinline__ void topk_insert_thread(unsigned long long* slots, in
   }
 }
 
-// topk_insert issued by a whole warp: the slots are read once in parallel
+// The same by a whole warp: the slots are read once in parallel
 // (one round instead of a chain of dependent reads) to find the first slot
 // not below the key; lane 0 then runs the compare-exchange chain from there.
 // All 32 lanes must call it with the same arguments.

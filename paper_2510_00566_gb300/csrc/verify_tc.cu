@@ -956,7 +956,6 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
       ChunkState cs;
       cs.start(nch, first_test);
       for (int l = first_test, l0 = 0;;) {
-        bool ok = true;
         uint32_t test = 0;
         for (int c = 0; c < nch; ++c)
           if (((cs.live >> c) & 1u) && cs.test_level(c) == l) test |= 1u << c;
@@ -1008,7 +1007,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
           set_query_terms(tid, fminf(tau, __ldcg(a.tau_seed + q)),
                           a.eps * a.qtail[(int64_t)q * (L + 1) + l + 1], sh.qterm);
         }
-        if ((bad = epi_or(!ok || failed(fail)))) break;
+        if ((bad = epi_or(failed(fail)))) break;
         const QTerms& qt = sh.qterm;
 #pragma unroll 1
         for (uint32_t m = test; m; m &= m - 1) {
@@ -1057,6 +1056,7 @@ __global__ void __launch_bounds__(NT, 2) verify_tc_kernel(const __grid_constant_
         section(2);
         if (l + 1 >= L) break;
         // the outcome of the level's tests: lane c looks at chunk c
+        bool ok = true;
         int n = 0;
         if (lane < S && ((test >> lane) & 1u)) {
           const uint32_t par = (tph >> lane) & 1u;
