@@ -11,11 +11,11 @@
 // for the exact re-ranking.  The id of a vector is its row.
 //
 // Search (refine_kernel, one CTA per query): Algorithm 1 seeds the heap with k
-// exact distances; the rest are refined level by level, eight lanes per
-// candidate, against the threshold of the moment with the margined separable
-// test of the IVF kernels.  A candidate that passes every level is re-ranked at
-// once on the original rows by its warp and inserted into the query's top-k in
-// shared memory.
+// exact distances; the rest are refined level by level with the margined
+// separable test of the IVF kernels, in rounds of 256 (a candidate per lane) or,
+// many queries of long rows, eight lanes per candidate.  Candidates that pass
+// every level are re-ranked on the original rows and inserted into the query's
+// top-k in shared memory.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -29,9 +29,9 @@
 namespace pano {
 namespace {
 
-constexpr int RT = 256;           // threads per query
-constexpr int RG = 8;             // lanes per candidate
+constexpr int RT = 256;           // threads per query; candidates per round
 constexpr int RW = RT / 32;
+static_assert(2 * RT == 512, "nine bits of hash");
 constexpr int kRefineMaxK = 1024;
 constexpr int kSeedScan = 2048;  // candidates ranked for the seed (shared memory)
 constexpr float kEval = 32.f * 5.9604645e-08f;  // evaluation slack of the separable test
@@ -99,10 +99,11 @@ __device__ __forceinline__ float sqrt_ratio_up_r(float tau, float inv_lb_up) {
   return __fmul_ru(__fmul_ru(y, rsqrtf(y)), 1.0f + 0x1p-19f);
 }
 
-// Partial product of coordinates [m0, m1) of a row by the eight lanes of a
+// Partial product of coordinates [m0, m1) of a row by the RG lanes of a
 // group (every lane of the group gets it; lanes of groups that are off pass
-// on = false and must call it too).  A group's lanes read 128 consecutive
-// bytes at a time.
+// on = false and must call it too).  Eight lanes read 128 consecutive bytes at a
+// time.
+template <int RG>
 __device__ __forceinline__ float group_dot(const float* qs, const float* x, int m0, int m1,
                                            bool vec, bool on, int t) {
   float acc = 0.f;
@@ -121,6 +122,7 @@ __device__ __forceinline__ float group_dot(const float* qs, const float* x, int 
         acc = fmaf(qv.w, xv.w, acc);
       }
     } else {
+#pragma unroll 4
       for (int j = m0 + t; j < m1; j += RG) acc = fmaf(qs[j], __ldg(x + j), acc);
     }
   }
@@ -130,14 +132,23 @@ __device__ __forceinline__ float group_dot(const float* qs, const float* x, int 
 }
 
 // Bound: gathered row segments (L2 / HBM): a candidate-level is one slice of a
-// scattered row.  Eight lanes per candidate read whole 128-byte lines of it (a
-// lane per row used half of every sector it fetched, one 16-byte load at a
-// time), and the four candidates of a warp go on independently: each group
-// takes its next candidate when its own dies, so no lane waits for another
-// candidate's levels and the threshold is always the current one (rounds of
-// 256 candidates ended in a block barrier each).  4,096 queries x 1,000
-// candidates of 960 coordinates, k = 10: 4.66 -> 2.23 ms.
+// scattered row.  Two forms (refine() chooses):
+//
+// GROUPS: eight lanes per candidate read whole 128-byte lines of it (a lane per
+// row uses half of every sector it fetches, one 16-byte load at a time), and
+// the four candidates of a warp go on independently: each group takes its next
+// candidate when its own dies, so no lane waits for another candidate's levels
+// and the threshold is always the current one.  What passes every level is
+// re-ranked at once by its warp.
+//
+// Otherwise: rounds of 256 candidates, one per lane, against the threshold that
+// the round began with; its survivors are re-ranked and inserted at its end, a
+// thread each, so that the insertions' chains overlap.  All of a block's
+// candidates are in flight at once, which a few queries or short rows need, and
+// the result of a relaxed bound does not depend on timing.
+template <bool GROUPS>
 __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
+  constexpr int RG = GROUPS ? 8 : 1;
   extern __shared__ __align__(16) unsigned char sm[];
   const int d = a.d, L = a.L, k = a.k, kp = a.kp;
   const int ns = min(kp, kSeedScan);
@@ -148,6 +159,12 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   __shared__ float qtl[65];
   __shared__ int s_next;
   __shared__ float s_tk;
+  // a round's survivors: ids, Eq. 3 bounds (the lower one becomes the distance)
+  __shared__ int32_t pid[GROUPS ? 1 : RT];
+  __shared__ float plb[GROUPS ? 1 : RT], pub[GROUPS ? 1 : RT];
+  __shared__ uint16_t keep[GROUPS ? 1 : RT];
+  __shared__ int32_t held[GROUPS ? 1 : 2 * RT];  // hash table of the round's survivors
+  __shared__ int s_np, s_nk;
   __shared__ unsigned long long s_dims, s_cands, s_rer;
   const int tid = threadIdx.x, warp = tid / 32, lane = tid & 31;
   const int grp = lane / RG, t = lane % RG;
@@ -155,9 +172,11 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   for (int i = tid; i < k; i += RT) topk[i] = kEmptyKey;
   for (int j = tid; j < d; j += RT) qs[j] = a.qt[q * d + j];
   for (int l = tid; l <= L; l += RT) qtl[l] = a.eps * a.qtail[q * (L + 1) + l];
+  if (!GROUPS)
+    for (int i = tid; i < 2 * RT; i += RT) held[i] = -1;
   if (tid == 0) {
     s_dims = s_cands = s_rer = 0;
-    s_next = 0;
+    s_next = s_np = s_nk = 0;
   }
   const float4 inf = a.qinfo[q];
   const float nq = inf.x, rq = inf.y, eq = inf.z, gs = a.gslack;
@@ -196,7 +215,7 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
     }
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-      p0[u] = group_dot(qs, a.xt + (on[u] ? id[u] : 0) * d, 0, m1, vec0, on[u], t);
+      p0[u] = group_dot<RG>(qs, a.xt + (on[u] ? id[u] : 0) * d, 0, m1, vec0, on[u], t);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int c = c0 + u * GPB + warp * (32 / RG) + grp;
@@ -235,63 +254,42 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   }
   __syncthreads();
 
-  // The other candidates, a group of eight lanes each.
+  // The other candidates.
   unsigned long long seen = kEmptyKey - 1;  // the k-th key that E and Hq stand for
   float E = 0.f, Hq = 0.f;
   unsigned n_cand = 0, n_rer = 0;
-  int64_t id = -1;    // the group's candidate (-1: none), its level and partial product
-  int l = 0;
+  int64_t id = -1;    // the group's candidate (-1: none) and its partial product
+  bool known = false;  // its first level's product is in p already
   float p = 0.f, rx = 0.f, exv = 0.f, Hx = 0.f;
-  bool open = true;   // the list is not exhausted
-  const unsigned gmask = 0xffu << (grp * RG);
-  while (true) {
-    // groups without a candidate take the next one of the list
-    if (id < 0 && open) {
-      while (true) {
-        int c = 0;
-        if (t == 0) c = atomicAdd(&s_next, 1);
-        c = __shfl_sync(gmask, c, grp * RG);
-        if (c >= kp) {
-          open = false;
-          break;
-        }
-        if (c < ns && akey[c] < 0.f) continue;  // a seed
-        const int64_t i = cl[c];
-        if (i < 0 || i >= a.n) {
-          if (t == 0) valid_id(i);
-          continue;
-        }
-        id = i;
-        const float nx = __ldg(a.xn2 + i);
-        exv = __ldg(a.ex + i);
-        rx = sqrtf(nx);
-        Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
-        l = 0;
-        p = 0.f;
-        if (t == 0) ++n_cand;
-        if (c < ns) {  // its first level is known
-          p = p0s[c];
-          l = -1;
-        }
-        break;
-      }
+  // takes entry c of the list, unless it is a seed or absent
+  auto take = [&](int c) {
+    if (c < ns && akey[c] < 0.f) return;
+    const int64_t i = cl[c];
+    if (i < 0 || i >= a.n) {
+      if (t == 0) valid_id(i);
+      return;
     }
-    __syncwarp();
+    id = i;
+    const float nx = __ldg(a.xn2 + i);
+    exv = __ldg(a.ex + i);
+    rx = sqrtf(nx);
+    Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
+    known = c < ns;
+    p = known ? p0s[c] : 0.f;
+    if (t == 0) ++n_cand;
+  };
+  auto threshold = [&](unsigned long long kth) {
+    if (kth == seen) return;
+    seen = kth;
+    const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
+    E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
+    Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
+  };
+  // one level of every group's candidate (a first level that is known is only
+  // tested); the next level's lines head for L2 meanwhile.  Clears id where the
+  // margined Eq. 3 test (separable form) prunes: LB > tau.
+  auto level = [&](int l) {
     const bool on = id >= 0;
-    if (!__any_sync(0xffffffffu, on)) break;
-    // (one value for the warp: the lanes of a group must decide alike)
-    const unsigned long long kth =
-        __shfl_sync(0xffffffffu, ld_volatile_u64(topk + k - 1), 0);
-    if (kth != seen) {
-      seen = kth;
-      const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
-      E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
-      Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
-    }
-    // one level of every group's candidate (a first level that is known is
-    // only tested); the next level's lines head for L2 meanwhile
-    const bool known = l < 0;
-    if (known) l = 0;
     const int a0 = on ? a.level_off[l] : 0, a1 = on ? a.level_off[l + 1] : 0;
     const float* x = a.xt + (on ? id : 0) * (int64_t)d;
     float tx = 0.f;
@@ -301,36 +299,105 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
       if (l + 1 < L && nxt < a.level_off[l + 2])
         asm volatile("prefetch.global.L2 [%0];" ::"l"(x + nxt));
     }
-    const float s = group_dot(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, on && !known, t);
-    bool done = false;
-    if (on) {
-      if (!known) {
-        p += s;
-        if (t == 0) dims += (unsigned long long)(a1 - a0);
-      }
-      // margined Eq. 3 (separable form): pruned when LB > tau
-      const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
-      if (P < Hq + Hx)
-        id = -1;
-      else if (++l == L)
-        done = true;
+    const float s = group_dot<RG>(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, on && !known, t);
+    if (!on) return;
+    if (!known) {
+      p += s;
+      if (t == 0) dims += (unsigned long long)(a1 - a0);
     }
-    // what passed every level: its exact distance, by the whole warp
-    for (unsigned m = __ballot_sync(0xffffffffu, done && t == 0); m; m &= m - 1) {
-      const int64_t i = __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
-      const float dist = exact_sqdist_warp_wide(qo, a.rows + i * d, d);
-      if (lane == 0) {
-        topk_insert_thread(topk, k, make_key(dist, (int32_t)i));
-        ++n_rer;
+    known = false;
+    const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
+    if (P < Hq + Hx) id = -1;
+  };
+  if (GROUPS) {
+    const unsigned gmask = ((1u << RG) - 1u) << (grp * RG);
+    bool open = true;  // the list is not exhausted
+    int l = 0;
+    while (true) {
+      while (id < 0 && open) {  // the next one of the list
+        int c = 0;
+        if (t == 0) c = atomicAdd(&s_next, 1);
+        c = __shfl_sync(gmask, c, grp * RG);
+        open = c < kp;
+        if (open) take(c);
+        l = 0;
       }
       __syncwarp();
+      if (!__any_sync(0xffffffffu, id >= 0)) break;
+      // (one value for the warp: the lanes of a group must decide alike)
+      threshold(__shfl_sync(0xffffffffu, ld_volatile_u64(topk + k - 1), 0));
+      level(l);
+      const bool done = id >= 0 && ++l == L;
+      // what passed every level: its exact distance, by the whole warp
+      for (unsigned m = __ballot_sync(0xffffffffu, done && t == 0); m; m &= m - 1) {
+        const int64_t i = __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
+        const float dist = exact_sqdist_warp_wide(qo, a.rows + i * d, d);
+        if (lane == 0) {
+          topk_insert_thread(topk, k, make_key(dist, (int32_t)i));
+          ++n_rer;
+        }
+        __syncwarp();
+      }
+      if (done) id = -1;
     }
-    if (done) id = -1;
+  } else {
+    for (int r0 = 0; r0 < kp; r0 += RT) {
+      threshold(ld_volatile_u64(topk + k - 1));
+      if (r0 + tid < kp) take(r0 + tid);
+      for (int l = 0; l < L && __any_sync(0xffffffffu, id >= 0); ++l) level(l);
+      if (id >= 0) {  // a repeat in the round is dropped (at most RT ids in 2 RT places)
+        uint32_t h = (uint32_t)id * 2654435761u >> 23;
+        int32_t was;
+        while ((was = atomicCAS(held + h, -1, (int32_t)id)) != -1 && was != (int32_t)id)
+          h = (h + 1) % (2 * RT);
+        if (was != -1) id = -1;
+      }
+      if (id >= 0) {  // its Eq. 3 bounds after the last level (C = 0)
+        const float nx = __ldg(a.xn2 + id), A = nq + nx - 2.f * p, S = rq + rx;
+        const float lr = sqrtf(fmaxf(A - gs * S * S, 0.f)) - (eq + exv);
+        const float ru = __fadd_ru(__fsqrt_ru(fmaxf(A + gs * S * S, 0.f)), eq + exv);
+        const int pos = atomicAdd(&s_np, 1);
+        pid[pos] = (int32_t)id;
+        plb[pos] = lr > 0.f ? lr * lr * a.lb_scale : 0.f;
+        pub[pos] = __fmul_ru(__fmul_ru(ru, ru), a.ub_scale);
+        id = -1;
+      }
+      __syncthreads();
+      // dropped: what k others have upper bounds below its lower bound
+      const int np = s_np;
+      bool in = tid < np;
+      if (in && np > k) {
+        const float lb = plb[tid];
+        int below = 0;
+        for (int o = 0; o < np && below < k; ++o) below += __fmul_ru(pub[o], 1.000001f) < lb;
+        in = below < k;
+      }
+      for (int i = tid; i < 2 * RT; i += RT) held[i] = -1;
+      if (in) keep[atomicAdd(&s_nk, 1)] = (uint16_t)tid;
+      __syncthreads();
+      // exact distances (a warp each), then the insertions (a thread each)
+      const int nk = s_nk;
+      for (int i = warp; i < nk; i += RW) {
+        const int v = keep[i];
+        const float dist = exact_sqdist_warp_wide(qo, a.rows + (int64_t)pid[v] * d, d);
+        if (lane == 0) plb[v] = dist;
+      }
+      __syncthreads();
+      if (tid < nk) topk_insert_thread(topk, k, make_key(plb[keep[tid]], pid[keep[tid]]));
+      if (tid == 0) {
+        n_rer += nk;
+        s_np = s_nk = 0;
+      }
+      __syncthreads();
+    }
   }
-  if (t == 0) {
+  n_cand = __reduce_add_sync(0xffffffffu, n_cand);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) dims += __shfl_xor_sync(0xffffffffu, dims, off);
+  if (lane == 0) {
     atomicAdd(&s_dims, dims);
     atomicAdd(&s_cands, (unsigned long long)n_cand);
-    if (lane == 0) atomicAdd(&s_rer, (unsigned long long)n_rer);
+    atomicAdd(&s_rer, (unsigned long long)n_rer);
   }
   __syncthreads();
   for (int i = tid; i < k; i += RT) {
@@ -493,9 +560,19 @@ int refine(const pano_index* ip, const float* queries, int64_t nq, const int64_t
   for (int l = 0; l <= L; ++l) a.level_off[l] = I.offs[l];
   const size_t smem =
       (size_t)((d + 3) & ~3) * 4 + (size_t)k * 8 + (size_t)std::min(kprime, kSeedScan) * 8;
-  PANO_CUDA(cudaFuncSetAttribute(refine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  // Groups pay where rows are long, few results keep the insertions short, and
+  // the queries fill the chip.  Rounds / groups, us a call, 1,000 candidates, k =
+  // 10: 600 queries of 1,536 coordinates (24 levels) 1,557 / 825, of 960 (16) 726 /
+  // 477, of 768 (12) 635 / 527, of 384 (6) 266 / 321; 152 queries of 960 355 / 460;
+  // 2,000 of 960 with k = 32 1,822 / 1,622, with k = 64 1,922 / 2,143.  Coordinates
+  // that are no multiple of 4 are read one by one: 2,000 of 129 818 / 1,959.
+  int sms = 0;
+  PANO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, I.device));
+  const bool groups = a.eps >= 1.f && k <= 32 && d % 4 == 0 && d >= 768 && nq >= 3 * sms;
+  auto kern = groups ? refine_kernel<true> : refine_kernel<false>;
+  PANO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)std::max<size_t>(smem, 48 * 1024)));
-  refine_kernel<<<(unsigned)nq, RT, smem, st>>>(a);
+  kern<<<(unsigned)nq, RT, smem, st>>>(a);
   PANO_CUDA(cudaGetLastError());
   int herr = 0;
   unsigned long long hst[3];
