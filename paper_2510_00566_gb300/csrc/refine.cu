@@ -254,80 +254,87 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
   }
   __syncthreads();
 
-  // The other candidates.
-  unsigned long long seen = kEmptyKey - 1;  // the k-th key that E and Hq stand for
-  float E = 0.f, Hq = 0.f;
   unsigned n_cand = 0, n_rer = 0;
-  int64_t id = -1;    // the group's candidate (-1: none) and its partial product
-  bool known = false;  // its first level's product is in p already
-  float p = 0.f, rx = 0.f, exv = 0.f, Hx = 0.f;
-  // takes entry c of the list, unless it is a seed or absent
-  auto take = [&](int c) {
-    if (c < ns && akey[c] < 0.f) return;
-    const int64_t i = cl[c];
-    if (i < 0 || i >= a.n) {
-      if (t == 0) valid_id(i);
-      return;
-    }
-    id = i;
-    const float nx = __ldg(a.xn2 + i);
-    exv = __ldg(a.ex + i);
-    rx = sqrtf(nx);
-    Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
-    known = c < ns;
-    p = known ? p0s[c] : 0.f;
-    if (t == 0) ++n_cand;
-  };
-  auto threshold = [&](unsigned long long kth) {
-    if (kth == seen) return;
-    seen = kth;
-    const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
-    E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
-    Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
-  };
-  // one level of every group's candidate (a first level that is known is only
-  // tested); the next level's lines head for L2 meanwhile.  Clears id where the
-  // margined Eq. 3 test (separable form) prunes: LB > tau.
-  auto level = [&](int l) {
-    const bool on = id >= 0;
-    const int a0 = on ? a.level_off[l] : 0, a1 = on ? a.level_off[l + 1] : 0;
-    const float* x = a.xt + (on ? id : 0) * (int64_t)d;
-    float tx = 0.f;
-    if (on) {
-      tx = __ldg(a.tails + id * (L + 1) + l + 1);
-      const int nxt = a1 + 32 * t;  // (128 bytes per lane)
-      if (l + 1 < L && nxt < a.level_off[l + 2])
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(x + nxt));
-    }
-    const float s = group_dot<RG>(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, on && !known, t);
-    if (!on) return;
-    if (!known) {
-      p += s;
-      if (t == 0) dims += (unsigned long long)(a1 - a0);
-    }
-    known = false;
-    const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
-    if (P < Hq + Hx) id = -1;
-  };
   if (GROUPS) {
-    const unsigned gmask = ((1u << RG) - 1u) << (grp * RG);
-    bool open = true;  // the list is not exhausted
+    // The other candidates, a group of eight lanes each.
+    unsigned long long seen = kEmptyKey - 1;  // the k-th key that E and Hq stand for
+    float E = 0.f, Hq = 0.f;
+    int64_t id = -1;    // the group's candidate (-1: none), its level and partial product
     int l = 0;
+    float p = 0.f, rx = 0.f, exv = 0.f, Hx = 0.f;
+    bool open = true;   // the list is not exhausted
+    const unsigned gmask = 0xffu << (grp * RG);
     while (true) {
-      while (id < 0 && open) {  // the next one of the list
-        int c = 0;
-        if (t == 0) c = atomicAdd(&s_next, 1);
-        c = __shfl_sync(gmask, c, grp * RG);
-        open = c < kp;
-        if (open) take(c);
-        l = 0;
+      // groups without a candidate take the next one of the list
+      if (id < 0 && open) {
+        while (true) {
+          int c = 0;
+          if (t == 0) c = atomicAdd(&s_next, 1);
+          c = __shfl_sync(gmask, c, grp * RG);
+          if (c >= kp) {
+            open = false;
+            break;
+          }
+          if (c < ns && akey[c] < 0.f) continue;  // a seed
+          const int64_t i = cl[c];
+          if (i < 0 || i >= a.n) {
+            if (t == 0) valid_id(i);
+            continue;
+          }
+          id = i;
+          const float nx = __ldg(a.xn2 + i);
+          exv = __ldg(a.ex + i);
+          rx = sqrtf(nx);
+          Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
+          l = 0;
+          p = 0.f;
+          if (t == 0) ++n_cand;
+          if (c < ns) {  // its first level is known
+            p = p0s[c];
+            l = -1;
+          }
+          break;
+        }
       }
       __syncwarp();
-      if (!__any_sync(0xffffffffu, id >= 0)) break;
+      const bool on = id >= 0;
+      if (!__any_sync(0xffffffffu, on)) break;
       // (one value for the warp: the lanes of a group must decide alike)
-      threshold(__shfl_sync(0xffffffffu, ld_volatile_u64(topk + k - 1), 0));
-      level(l);
-      const bool done = id >= 0 && ++l == L;
+      const unsigned long long kth =
+          __shfl_sync(0xffffffffu, ld_volatile_u64(topk + k - 1), 0);
+      if (kth != seen) {
+        seen = kth;
+        const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
+        E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
+        Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
+      }
+      // one level of every group's candidate (a first level that is known is
+      // only tested); the next level's lines head for L2 meanwhile
+      const bool known = l < 0;
+      if (known) l = 0;
+      const int a0 = on ? a.level_off[l] : 0, a1 = on ? a.level_off[l + 1] : 0;
+      const float* x = a.xt + (on ? id : 0) * (int64_t)d;
+      float tx = 0.f;
+      if (on) {
+        tx = __ldg(a.tails + id * (L + 1) + l + 1);
+        const int nxt = a1 + 32 * t;  // (128 bytes per lane)
+        if (l + 1 < L && nxt < a.level_off[l + 2])
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(x + nxt));
+      }
+      const float s = group_dot<RG>(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, on && !known, t);
+      bool done = false;
+      if (on) {
+        if (!known) {
+          p += s;
+          if (t == 0) dims += (unsigned long long)(a1 - a0);
+        }
+        // margined Eq. 3 (separable form): pruned when LB > tau
+        const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
+        if (P < Hq + Hx)
+          id = -1;
+        else if (++l == L)
+          done = true;
+      }
       // what passed every level: its exact distance, by the whole warp
       for (unsigned m = __ballot_sync(0xffffffffu, done && t == 0); m; m &= m - 1) {
         const int64_t i = __shfl_sync(0xffffffffu, id, __ffs(m) - 1);
@@ -341,6 +348,48 @@ __global__ void __launch_bounds__(RT) refine_kernel(const RefineArgs a) {
       if (done) id = -1;
     }
   } else {
+    // The other candidates, one per lane, RT at a time.
+    float E = 0.f, Hq = 0.f;
+    int64_t id = -1;     // the lane's candidate (-1: none) and its partial product
+    bool known = false;
+    float p = 0.f, rx = 0.f, exv = 0.f, Hx = 0.f;
+    // takes entry c of the list, unless it is a seed or absent
+    auto take = [&](int c) {
+      if (c < ns && akey[c] < 0.f) return;
+      const int64_t i = cl[c];
+      if (i < 0 || i >= a.n) {
+        valid_id(i);
+        return;
+      }
+      id = i;
+      const float nx = __ldg(a.xn2 + i);
+      exv = __ldg(a.ex + i);
+      rx = sqrtf(nx);
+      Hx = 0.5f * (nx - gs * nx - exv * exv - kEval * (rx + exv) * (rx + exv));
+      known = c < ns;  // its first level is only to be tested
+      p = known ? p0s[c] : 0.f;
+      ++n_cand;
+    };
+    auto threshold = [&](unsigned long long kth) {
+      const float tau = kth == kEmptyKey ? INFINITY : __fmul_ru(key_dist(kth), 1.000001f);
+      E = __fadd_ru(eq, tau == INFINITY ? 1e18f : sqrt_ratio_up_r(tau, a.inv_lb_up));
+      Hq = 0.5f * (nq - gs * nq - E * E - kEval * (rq + E) * (rq + E));
+    };
+    // Level l; the next one heads for L2 meanwhile.  Clears id where the margined
+    // Eq. 3 test (separable form) prunes: LB > tau.
+    auto level = [&](int l) {
+      if (id < 0) return;
+      const int a0 = a.level_off[l], a1 = a.level_off[l + 1];
+      const float* x = a.xt + id * (int64_t)d;
+      const float tx = __ldg(a.tails + id * (L + 1) + l + 1);
+      if (l + 1 < L) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + a1));
+      if (l > 0 || !known) {
+        p += group_dot<1>(qs, x, a0, a1, vec_d && ((a0 | a1) & 3) == 0, true, 0);
+        dims += (unsigned long long)(a1 - a0);
+      }
+      const float P = fmaf(E, exv, fmaf(gs * rq, rx, fmaf(qtl[l + 1], tx, p)));
+      if (P < Hq + Hx) id = -1;
+    };
     for (int r0 = 0; r0 < kp; r0 += RT) {
       threshold(ld_volatile_u64(topk + k - 1));
       if (r0 + tid < kp) take(r0 + tid);

@@ -39,7 +39,7 @@ def test_many_results(kprime, k, nq):
     check_topk(X, Q, ids.cpu().numpy(), dist.cpu().numpy(), want_i, want_d, k)
 
 
-@pytest.mark.parametrize("d,nq", [(96, 9), (960, 9), (960, 400)])
+@pytest.mark.parametrize("d,nq", [(96, 9), (960, 9), (960, 480)])
 @pytest.mark.parametrize("kprime", [100, 700])
 def test_lists_of_repeats(d, nq, kprime):
     # every id three to six times: repeats are no others that rule a candidate out
@@ -56,6 +56,33 @@ def test_lists_of_repeats(d, nq, kprime):
             o = np.lexsort((c, e))[:k]
             want_i[i, :len(o)], want_d[i, :len(o)] = c[o], e[o]
         check_topk(X, Q, ids.cpu().numpy(), dist.cpu().numpy(), want_i, want_d, k)
+
+
+@pytest.mark.parametrize("widths", [[64] * 12, [4, 764], [100, 68, 632], [32] * 25, [256] * 4])
+@pytest.mark.parametrize("kprime,k", [(1, 1), (5, 10), (37, 3), (300, 32), (2_500, 10)])
+def test_groups_answer_as_rounds(widths, kprime, k):
+    # many queries of long rows take groups of eight lanes, a few of them rounds
+    d, nq = sum(widths), 480
+    s = synth.scaled(1, n=3_000, n_queries=nq, nlist=1, n_clusters=0, d=d, n_levels=1, decay=4.0 / d)
+    w = synth.generate(s)
+    t = pano.panorama_transform_import(np.eye(d), np.zeros(d), np.ones(d))
+    idx = pano.panorama_build_flat(t, w.X.to(DEV), level_widths=widths)
+    rng = np.random.default_rng(kprime)
+    cand = np.stack([rng.permutation(3_000)[:kprime] for _ in range(nq)]).astype(np.int64)
+    cand[:, 11::17] = -1
+    q, c = w.Q.to(DEV), torch.from_numpy(cand).to(DEV)
+    ids, dist = idx.refine(q, c, k)
+    for rows in (slice(0, 40), slice(440, 480)):
+        a, b = idx.refine(q[rows].contiguous(), c[rows].contiguous(), k)
+        assert torch.equal(a, ids[rows]) and torch.equal(b, dist[rows])
+    X, Q = w.X.numpy(), w.Q.numpy()
+    for i in (0, 77, 479):
+        ci = np.unique(cand[i][cand[i] >= 0])
+        e = ((X[ci].astype(np.float64) - Q[i]) ** 2).sum(1)
+        o = np.lexsort((ci, e))[:k]
+        assert np.array_equal(ids[i].cpu().numpy()[:len(o)], ci[o])
+        assert np.allclose(dist[i].cpu().numpy()[:len(o)], e[o], rtol=1e-5, atol=0)
+        assert np.all(ids[i].cpu().numpy()[len(o):] == -1)
 
 
 @pytest.mark.parametrize("epsilon", [0.9, 0.6, 0.3])
