@@ -1,6 +1,7 @@
 // Device helpers shared by the library's kernels: bulk-async (TMA engine)
 // copies with mbarrier completion, bounded waits, (distance, id) keys and the
-// lock-free k-smallest insertion used for the running top-k.
+// two lock-free ways they enter a query's running top-k: chains through sorted
+// slots, and replacement of the largest of unsorted ones.
 #pragma once
 
 #include <cuda_runtime.h>

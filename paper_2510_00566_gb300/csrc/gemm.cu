@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(NT, 2) gemm_nt64_kernel(int M, int N, int K,
 
 // A few rows (kStoreAny, M <= kRowsMax): one warp per (row, column), the lanes
 // along K, so that every SM has a part of B to read; the 128 x 64 tiles left all
-// but N / 64 of them idle (one query of 960: 298 us a search, 244 so with
-// the seeds below 152 queries).  A product
-// passes through ceil(K / 32) + 6 roundings at most, fewer than in the tiles.
+// but N / 64 of them idle (one query of 960: 298 us a search, 244 so and with
+// sixteen warps for the seeds).  A product passes through ceil(K / 32) + 6
+// roundings at most, fewer than in the tiles.
 constexpr int kRowsMax = 8;
 
 __global__ void __launch_bounds__(NT) gemm_rows_kernel(int N, int K, const float* __restrict__ A,

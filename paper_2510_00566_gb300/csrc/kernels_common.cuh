@@ -398,7 +398,7 @@ struct RowBounds {
 // All results are those of FP64 sums, rounded once to FP32, but the sums are
 // compensated FP32: FP64 arithmetic per element was most of the packers' time
 // (a warp's FP64 instruction takes 16 cycles; 500k x 384 BF16 rows: 11.3 ms,
-// 3.0 so).  Where a sum's error (a few 1e-12 of it) could move one of the
+// 3.4 so).  Where a sum's error (a few 1e-12 of it) could move one of the
 // row's results to another FP32 number, the row is summed again in FP64.
 template <class Stored, class Err, class Dev, class AddErr, class AddDev>
 __device__ __forceinline__ RowBounds row_bounds(int d, int L, const int32_t* __restrict__ level_off,

@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(256) pack_fp8_kernel(
 //       the last level filter and defer the survivors; then the accumulators
 //       go back to the MMA thread, which has the next item's tiles waiting.
 //
-// What bounds it: instruction issue and latency of the epilogue (about 45 % of
-// the issue slots; tensor pipe 18 %, L2 21 %, ncu on 1.5M x 768), so its code is
+// What bounds it: instruction issue and latency of the epilogue (44 % of the
+// issue slots; tensor pipe 17 %, L2 21 %, ncu on 500k x 768), so its code is
 // kept small (the roles share one instruction cache: survivors unrolled over
 // 32 slots cost 15 %) and its tests run two queries per instruction.  Against
 // the same work in lockstep, a CTA barrier per level and the query split redone
